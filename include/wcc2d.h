@@ -48,8 +48,11 @@ extern "C" {
 
 /* Options.  wcc2d_default_options fills: precision = WCC_FP64, limiter = 1,
  * alpha = 2, eps = 1e-40 (Eq. 2D2ndOrderWeights), gamma = 1.4, ax = ay = 1,
- * rows_per_cta = 16 (new rows one CTA marches through), cuda_stream = NULL
- * (the handle creates its own non-blocking stream).  precision is WCC_FP64,
+ * rows_per_cta = 16, cuda_stream = NULL (the handle creates its own
+ * non-blocking stream).  rows_per_cta is the number of new rows one CTA
+ * marches through; the default, 16, stands for a height (and strip width)
+ * picked from the mesh, any other value is taken as it is.  The results do not
+ * depend on it.  precision is WCC_FP64,
  * WCC_FP32 (every value and operation in float) or WCC_FP32_MIXED (float
  * arithmetic, with the cell average, the leading flux terms and the vertex
  * point values in float-float, so that the averages keep about 48 bits). */
@@ -119,7 +122,7 @@ int wcc2d_get_dt_history(wcc2d_handle h, double* dts, int64_t cap, int64_t* n);
 int wcc2d_synchronize(wcc2d_handle h);
 
 /* Autotuner of the strip height: times rows_per_cta = 8 .. 24 (13
- * candidates; the count of CTAs, and so how full the last wave of resident
+ * candidates, 16 standing for the height picked from the mesh; the count of CTAs, and so how full the last wave of resident
  * CTAs is, changes with it) on the handle's own current stage at CFL number
  * cfl, one warm-up and four timed half-steps each (CUDA events on the
  * handle's stream), keeps the fastest in the handle's options and reports it

@@ -17,6 +17,8 @@ using namespace wcc2d;
 
 namespace {
 thread_local std::string g_create_error2d;
+// The default strip height: stands for the height picked from the mesh (plan_strips).
+constexpr int kDefaultRows2D = 16;
 }
 
 struct wcc2d_ctx {
@@ -27,6 +29,7 @@ struct wcc2d_ctx {
     int64_t nx = 0, ny = 0;
     double x0 = 0, x1 = 1, y0 = 0, y1 = 1, dx = 1, dy = 1;
     wcc2d_options opt{};
+    StripPlan plan[2] = {{16, 0}, {16, 0}};  // strips picked for the new stage of either parity
     Law2D law{};
     cudaStream_t stream = nullptr;
     bool own_stream = false;
@@ -110,6 +113,22 @@ int read_state(wcc2d_ctx* h, DevState2D* out) {
     return WCC_OK;
 }
 
+// Strips of the half-steps onto the stage of each parity.
+cudaError_t plan_launches(wcc2d_ctx* h) {
+    int sms = 0, resident = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+    if (e != cudaSuccess) return e;
+    Step2D q{};
+    q.resident = &resident;
+    e = h->mixed ? launch_halfstep2d_mx(h->system, h->P, q, h->stream)
+                 : launch_halfstep2d(h->system, h->P, h->fp32 != 0, q, h->stream);
+    if (e != cudaSuccess) return e;
+    const int tw = strip_threads(h->system, h->P, h->fp32 != 0, h->mixed != 0);
+    for (int p = 0; p < 2; ++p)
+        h->plan[p] = plan_strips(tw, !h->fp32, std::max(1, resident), sms, (int)stage_cells_x(h, p), (int)stage_cells_y(h, p));
+    return cudaSuccess;
+}
+
 int conv_grid(long long n) { return (int)std::min<long long>((n + 255) / 256, 152LL * 16); }
 
 }  // namespace
@@ -126,7 +145,7 @@ void wcc2d_default_options(wcc2d_options* o) {
     o->gamma = 1.4;
     o->ax = 1.0;
     o->ay = 1.0;
-    o->rows_per_cta = 16;
+    o->rows_per_cta = kDefaultRows2D;
     o->cuda_stream = nullptr;
 }
 
@@ -216,7 +235,8 @@ int wcc2d_create(wcc2d_handle* out, int system, int64_t nx, int64_t ny, int P, c
         delete h;
         return fail2(nullptr, WCC_E_NOMEM, m);
     }
-    e = cudaStreamSynchronize(h->stream);
+    e = plan_launches(h);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) {
         release(h);
         delete h;
@@ -302,7 +322,11 @@ int launch_one(wcc2d_ctx* h, double dt_given, double cfl) {
     a.ny_new = (int)stage_cells_y(h, h->parity ^ 1);
     a.parity = h->parity;
     a.bc = h->bc;
-    a.rows_per_cta = h->opt.rows_per_cta;
+    const StripPlan& plan = h->plan[h->parity ^ 1];
+    const bool planned = h->opt.rows_per_cta == kDefaultRows2D;
+    a.rows_per_cta = planned ? plan.rows : h->opt.rows_per_cta;
+    a.strip = planned ? plan.strip : 0;
+    a.resident = nullptr;
     a.dx = h->dx;
     a.dy = h->dy;
     a.inv_dx = 1.0 / h->dx;

@@ -47,6 +47,8 @@ struct Step2D {
     DevState2D* st;
     double* hist;
     long long hist_cap;
+    int strip;      // FP64: threads per CTA, 32 or 0 (the degree's full width, strip_width)
+    int* resident;  // host: not null asks for the kernel's resident CTAs per SM instead of a launch
 };
 
 __device__ __forceinline__ int parent_index(int j, int n_old, int bc) {
@@ -318,15 +320,62 @@ constexpr int strip_width() {
     return tw;
 }
 
-// Launch one half-step of system SYS at degree P in type T.
-template <int SYS, int P, class T>
-cudaError_t launch_halfstep2d_t(const Step2D& a, cudaStream_t stream) {
-    constexpr int TW = strip_width<SYS, P, T>();
+// Strip height and width (0: full) of a half-step.
+struct StripPlan {
+    int rows, strip;
+};
+
+// Strip height for a mesh, from a model of the time: a CTA marches rows + 1
+// parent rows and rows new rows, about equally dear (2 rows + 1 units), and
+// the CTAs run in waves of `slots`, so the time goes as
+// ceil(CTAs / slots) (2 rows + 1).  The minimum over the heights trades the
+// parent row that neighbouring strips both expand against SMs left idle.
+// FP32: slots are the resident CTAs.  Measured (FP32-mixed Euler, P = 3):
+// 1024 x 1024 0.259 ms at 16 rows (704 CTAs on 608 slots, two waves) against
+// 0.200 ms at the 19 rows this picks (594 CTAs, one wave); sweeps of the
+// height at 400, 700 and 1024 cells a side found nothing faster than its pick.
+// FP64: a warp's FP64 instruction takes its scheduler's share of the pipe for
+// 64 cycles whatever else runs, so the slots are the 4 schedulers per SM and
+// the unit is the warp; strips of one warp are taken where they shorten the
+// longest chain (192 x 192 Euler, P = 3: 48 CTAs of 64 threads and 16 rows
+// 1.87 ms, 455 of 32 threads and 3 rows 0.42 ms).
+inline StripPlan plan_strips(int tw, bool fp64, int resident, int sms, int nx_new, int ny_new) {
+    StripPlan best{16, 0};
+    double best_cost = 1e300;
+    for (int width = tw; width >= 32; width = width > 32 && fp64 ? 32 : 0) {
+        const long long strips = (nx_new + width - 2) / (width - 1);
+        for (int rows = 48; rows >= 1; --rows) {
+            if (rows > ny_new) continue;
+            long long units = strips * ((ny_new + rows - 1) / rows);
+            if (fp64) units *= width / 32;
+            const long long slots = (long long)sms * (fp64 ? 4 : resident);
+            const double cost = (double)((units + slots - 1) / slots) * (2 * rows + 1);
+            if (cost < best_cost) {
+                best_cost = cost;
+                best = StripPlan{rows, width == tw ? 0 : width};
+            }
+        }
+    }
+    return best;
+}
+
+template <int SYS, int P, class T, int TW>
+cudaError_t launch_strips2d(const Step2D& a, cudaStream_t stream) {
     constexpr size_t smem = ring_bytes<T, TW>(record_fields<SYS, P>());
     static_assert(smem <= 48 * 1024 - 256, "the shared ring and the static shared words must fit without the opt-in attribute");
+    if (a.resident) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(a.resident, halfstep2d<SYS, P, T, TW>, TW, smem);
     const dim3 grid((a.nx_new + TW - 2) / (TW - 1), (a.ny_new + a.rows_per_cta - 1) / a.rows_per_cta);
     halfstep2d<SYS, P, T, TW><<<grid, TW, smem, stream>>>(a);
     return cudaGetLastError();
+}
+
+// Launch one half-step of system SYS at degree P in type T.
+template <int SYS, int P, class T>
+cudaError_t launch_halfstep2d_t(const Step2D& a, cudaStream_t stream) {
+    if constexpr (sizeof(T) == 8) {
+        if (a.strip == 32) return launch_strips2d<SYS, P, T, 32>(a, stream);
+    }
+    return launch_strips2d<SYS, P, T, strip_width<SYS, P, T>()>(a, stream);
 }
 
 template <int SYS, class T>
@@ -375,6 +424,20 @@ constexpr int strip_width_mx() {
     int tw = 128;
     while (tw > 32 && ring_bytes<float, 1>(record_fields_mx<SYS, P>()) * tw > 48 * 1024 - 256) tw -= 32;
     return tw;
+}
+
+// Threads per CTA of a kernel's full-width strips (host).
+inline int strip_threads(int system, int P, bool fp32, bool mixed) {
+    auto width = [&](auto sys) {
+        constexpr int S = decltype(sys)::value;
+        auto at = [&](auto pc) {
+            constexpr int Q = decltype(pc)::value;
+            return mixed ? strip_width_mx<S, Q>() : fp32 ? strip_width<S, Q, float>() : strip_width<S, Q, double>();
+        };
+        return P == 1 ? at(std::integral_constant<int, 1>{}) : P == 2 ? at(std::integral_constant<int, 2>{})
+                                                                      : at(std::integral_constant<int, 3>{});
+    };
+    return system == EULER ? width(std::integral_constant<int, EULER>{}) : width(std::integral_constant<int, ADVECTION>{});
 }
 
 template <int TW, int NV, int NQ1>
@@ -630,6 +693,7 @@ cudaError_t launch_halfstep2d_mx_t(const Step2D& a, cudaStream_t stream) {
     constexpr int TW = strip_width_mx<SYS, P>();
     constexpr size_t smem = ring_bytes<float, TW>(record_fields_mx<SYS, P>());
     static_assert(smem <= 48 * 1024 - 256, "the shared ring and the static shared words must fit without the opt-in attribute");
+    if (a.resident) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(a.resident, halfstep2d_mx<SYS, P, TW>, TW, smem);
     const dim3 grid((a.nx_new + TW - 2) / (TW - 1), (a.ny_new + a.rows_per_cta - 1) / a.rows_per_cta);
     halfstep2d_mx<SYS, P, TW><<<grid, TW, smem, stream>>>(a);
     return cudaGetLastError();
