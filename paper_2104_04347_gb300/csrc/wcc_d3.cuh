@@ -1,0 +1,119 @@
+// wcc_d3.cuh -- FP64 arithmetic in three-register fused multiply-adds.
+//
+// GB300's FP64 pipe takes a warp instruction every 16 SM cycles when all
+// three operands of a DFMA come from general registers, and every 19 when
+// an operand is missing (DADD, DMUL) or is a constant, an immediate or a
+// uniform register (measured with chains of each form, 4 to 16 warps per SM;
+// the FP64 kernels' own average was 18.5).  The FP64 kernels are bound by
+// that pipe, so they compute with this type: a + b is fma(a, 1, b), a b is
+// fma(a, b, -0), and 1, -0 and the scheme's constants are general registers.
+// Both forms round once, exactly as the addition and the product (signed
+// zeros included: x + -0 is x for either zero).
+//
+// A constant stays in a general register only if the compiler cannot know its
+// value: its bits are combined with a zero that depends on the lane and on
+// a word of constant memory, with one integer operation per half (the integer
+// pipe is idle here) and nothing on the FP64 pipe.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace wcc {
+
+static __constant__ unsigned k_opaque_mask = 0u;
+
+__device__ __forceinline__ unsigned opaque_zero() {
+    unsigned lane;
+    asm("mov.u32 %0, %%laneid;" : "=r"(lane));
+    return lane & k_opaque_mask;
+}
+
+struct d3 {
+    double v;
+    __device__ __forceinline__ d3() {}
+    // any double as a value in general registers (constants included)
+    __device__ __forceinline__ explicit d3(double x) {
+        const unsigned z = opaque_zero();
+        v = __hiloint2double((int)((unsigned)__double2hiint(x) ^ z), (int)((unsigned)__double2loint(x) ^ z));
+    }
+    __device__ __forceinline__ explicit d3(float x) : d3((double)x) {}
+    __device__ __forceinline__ explicit d3(int x) : d3((double)x) {}
+    static __device__ __forceinline__ d3 reg(double x) {  // already in a register (a load)
+        d3 r;
+        r.v = x;
+        return r;
+    }
+};
+
+__device__ __forceinline__ d3 operator-(d3 a) { return d3::reg(-a.v); }
+__device__ __forceinline__ d3 fma(d3 a, d3 b, d3 c) { return d3::reg(::fma(a.v, b.v, c.v)); }
+__device__ __forceinline__ d3 operator+(d3 a, d3 b) { return d3::reg(::fma(a.v, d3(1.0).v, b.v)); }
+__device__ __forceinline__ d3 operator-(d3 a, d3 b) { return d3::reg(::fma(a.v, d3(1.0).v, -b.v)); }
+__device__ __forceinline__ d3 operator*(d3 a, d3 b) { return d3::reg(::fma(a.v, b.v, d3(-0.0).v)); }
+__device__ __forceinline__ d3& operator+=(d3& a, d3 b) { a = a + b; return a; }
+__device__ __forceinline__ d3& operator*=(d3& a, d3 b) { a = a * b; return a; }
+__device__ __forceinline__ d3 fabs(d3 a) { return d3::reg(::fabs(a.v)); }
+
+// a > 0 (false for NaN), on the integer pipe
+__device__ __forceinline__ bool all_pos(d3 a) {
+    const long long b = __double_as_longlong(a.v);
+    return b > 0 && b <= 0x7ff0000000000000ll;
+}
+// NaN / Inf test on the exponent bits
+__device__ __forceinline__ bool not_finite(d3 x) { return (__double2hiint(x.v) & 0x7ff00000) == 0x7ff00000; }
+
+// Exponent between 2^-1000 and 2^1000: where the estimates below are normal
+// and their residuals exact to rounding.  Everything else (zeros, infinities,
+// NaN, extreme values, negative roots) takes the compiler's operations.
+__device__ __forceinline__ bool mid_range(double x) {
+    const unsigned e = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
+    return e - 23u <= 2000u;
+}
+static __device__ __noinline__ double recip_any(double x) { return 1.0 / x; }
+static __device__ __noinline__ double sqrt_any(double x) { return ::sqrt(x); }
+
+// 1/x: the special-function unit's estimate y (about 20 bits) and one step of
+// the cubic iteration y (1 + e + e^2), e = 1 - x y, whose remaining error is
+// e^3 (2^-60): three DFMAs, one rounding in the last place that matters.
+__device__ __forceinline__ d3 recip(d3 x) {
+    if (mid_range(x.v)) {
+        double y;
+        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x.v));
+        const d3 y0 = d3::reg(y);
+        const d3 e = fma(-x, y0, d3(1.0));
+        return fma(y0, fma(e, e, e), y0);
+    }
+    return d3::reg(recip_any(x.v));
+}
+
+// the limiter's weights for an exponent other than 2
+__device__ __forceinline__ d3 pow_any(d3 a, double p) { return d3::reg(::pow(a.v, p)); }
+__device__ __forceinline__ d3 div_any(d3 a, d3 b) { return d3::reg(a.v / b.v); }
+
+// half of a mid-range value: the exponent less one
+__device__ __forceinline__ d3 half_of(d3 a) {
+    return d3::reg(__hiloint2double(__double2hiint(a.v) - 0x100000, __double2loint(a.v)));
+}
+
+// sqrt(x) for a positive x, and half its reciprocal: from the estimate y of
+// 1/sqrt(x) (about 20 bits), e = 1 - x y^2 and (1 - e)^(-1/2) = 1 + e/2 +
+// 3 e^2/8 + ... (the next term is below 2^-60); the root is corrected once by
+// its own residual x - g^2.
+__device__ __forceinline__ d3 sqrt_half_rsqrt(d3 x, d3& half_rsqrt) {
+    if (mid_range(x.v) && __double2hiint(x.v) > 0) {
+        double y;
+        asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x.v));
+        const d3 y0 = d3::reg(y), h = x * y0;
+        const d3 e = fma(-h, y0, d3(1.0));
+        const d3 t = e * fma(d3(0.375), e, d3(0.5));
+        const d3 yh = half_of(y0);
+        half_rsqrt = fma(yh, t, yh);
+        const d3 g = fma(h, t, h);
+        return fma(fma(-g, g, x), half_rsqrt, g);
+    }
+    const double c = sqrt_any(x.v);
+    half_rsqrt = d3::reg(0.5 * recip_any(c));
+    return d3::reg(c);
+}
+
+}  // namespace wcc

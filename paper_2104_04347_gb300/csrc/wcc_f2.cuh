@@ -11,6 +11,8 @@
 
 #include <type_traits>
 
+#include "wcc_d3.cuh"
+
 namespace wcc {
 
 // keep the scalar math overloads visible next to the paired ones below
@@ -66,7 +68,7 @@ __device__ __forceinline__ f2 rsqrt_approx(f2 a) { return f2(rsqrtf(a.v.x), rsqr
 
 // Helpers the generic scheme code uses for every real type.
 template <class R>
-constexpr bool is_f64 = std::is_same<R, double>::value;
+constexpr bool is_f64 = std::is_same<R, double>::value || std::is_same<R, d3>::value;
 
 __device__ __forceinline__ bool all_pos(double a) { return a > 0.0; }
 __device__ __forceinline__ bool all_pos(float a) { return a > 0.f; }

@@ -142,23 +142,23 @@ __global__ void __launch_bounds__(kThreads) halfstep_fp64(const StepArgs args) {
     // ---- phase 1: parent record of parent slot t
     {
         const long long p = parent_index(first_new + t - (args.parity ? 1 : 0), args.n_old, args.bc);
-        double c[NV][K];
+        d3 c[NV][K];
         sfor<0, NV>([&](auto V) {
             constexpr int v = decltype(V)::value;
             sfor<0, K>([&](auto Ki) {
                 constexpr int k = decltype(Ki)::value;
-                c[v][k] = __ldg(args.in64 + (long long)(v * K + k) * args.pitch + p);
+                c[v][k] = d3::reg(__ldg(args.in64 + (long long)(v * K + k) * args.pitch + p));
             });
         });
-        ParentRecord<SYS, P, double> r;
-        parent_record<SYS, P, double>(c, lam, args, r);
+        ParentRecord<SYS, P, d3> r;
+        parent_record<SYS, P, d3>(c, d3(lam), args, r);
         sfor<0, NV>([&](auto V) {
             constexpr int v = decltype(V)::value;
-            rec[v][t] = r.A[v];
-            rec[NV + v][t] = r.B[v];
+            rec[v][t] = r.A[v].v;
+            rec[NV + v][t] = r.B[v].v;
             sfor<0, K>([&](auto Ki) {
                 constexpr int k = decltype(Ki)::value;
-                rec[2 * NV + v * K + k][t] = r.vtx[v][k];
+                rec[2 * NV + v * K + k][t] = r.vtx[v][k].v;
             });
         });
     }
@@ -169,35 +169,35 @@ __global__ void __launch_bounds__(kThreads) halfstep_fp64(const StepArgs args) {
     double speed = 0.0;
     unsigned err = 0u;
     if (t < kTile && i < args.n_new) {
-        double e[NV][K], ubar[NV], vl[NV], vr[NV];
+        d3 e[NV][K], ubar[NV], vl[NV], vr[NV];
         sfor<0, NV>([&](auto V) {
             constexpr int v = decltype(V)::value;
-            double vL[K], vR[K];
+            d3 vL[K], vR[K];
             sfor<0, K>([&](auto Ki) {
                 constexpr int k = decltype(Ki)::value;
-                vL[k] = rec[2 * NV + v * K + k][t];
-                vR[k] = rec[2 * NV + v * K + k][t + 1];
+                vL[k] = d3::reg(rec[2 * NV + v * K + k][t]);
+                vR[k] = d3::reg(rec[2 * NV + v * K + k][t + 1]);
             });
-            ubar[v] = rec[v][t] + rec[NV + v][t + 1];
+            ubar[v] = d3::reg(rec[v][t]) + d3::reg(rec[NV + v][t + 1]);
             vl[v] = vL[0];
             vr[v] = vR[0];
-            derivatives_and_point_value<P, double>(ubar[v], vL, vR, e[v]);
+            derivatives_and_point_value<P, d3>(ubar[v], vL, vR, e[v]);
         });
 
         if (args.limiter) {
             if constexpr (NV == 1) {
-                limit_scalar<P, double>(e[0], ubar[0], vl[0], vr[0], args);
+                limit_scalar<P, d3>(e[0], ubar[0], vl[0], vr[0], args);
             } else {
                 // Sec. 4: limit characteristic variables L(ubar) U, map back with R(ubar).
-                EulerChar<double> E;
-                if (!euler_char<double>(ubar, args.gamma, E)) err |= ERR_POSITIVITY;
-                double ce[3][K], cub[3], cvl[3], cvr[3];
+                EulerChar<d3> E;
+                if (!euler_char<d3>(ubar, d3(args.gamma), E)) err |= ERR_POSITIVITY;
+                d3 ce[3][K], cub[3], cvl[3], cvr[3];
                 E.left(ubar[0], ubar[1], ubar[2], cub);
                 E.left(vl[0], vl[1], vl[2], cvl);
                 E.left(vr[0], vr[1], vr[2], cvr);
                 sfor<0, K>([&](auto Ki) {
                     constexpr int k = decltype(Ki)::value;
-                    double w[3];
+                    d3 w[3];
                     E.left(e[0][k], e[1][k], e[2][k], w);
                     ce[0][k] = w[0];
                     ce[1][k] = w[1];
@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(kThreads) halfstep_fp64(const StepArgs args) {
                 });
                 sfor<0, 3>([&](auto Ii) {
                     constexpr int r = decltype(Ii)::value;
-                    limit_scalar<P, double>(ce[r], cub[r], cvl[r], cvr[r], args);
+                    limit_scalar<P, d3>(ce[r], cub[r], cvl[r], cvr[r], args);
                 });
                 sfor<0, K>([&](auto Ki) {
                     constexpr int k = decltype(Ki)::value;
@@ -220,13 +220,13 @@ __global__ void __launch_bounds__(kThreads) halfstep_fp64(const StepArgs args) {
             sfor<0, K>([&](auto Ki) {
                 constexpr int k = decltype(Ki)::value;
                 bad |= not_finite(e[v][k]);
-                __stcs(args.out64 + (long long)(v * K + k) * args.pitch + i, e[v][k]);
+                __stcs(args.out64 + (long long)(v * K + k) * args.pitch + i, e[v][k].v);
             });
         });
         if (bad) err |= ERR_NONFINITE;
-        double u0[NV];
+        d3 u0[NV];
         sfor<0, NV>([&](auto V) { u0[decltype(V)::value] = e[decltype(V)::value][0]; });
-        speed = wave_speed<SYS, double>(u0, args, err);
+        speed = wave_speed<SYS, d3>(u0, args, err).v;
     }
     finish_halfstep<double>(speed, err, dt, args);
 }
@@ -240,10 +240,10 @@ __global__ void __launch_bounds__(256) stage_speed(const double* u0planes, long 
     unsigned err = 0u;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
-        double u0[NV];
+        d3 u0[NV];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) u0[v] = u0planes[v * var_stride + i];
-        double s = wave_speed<SYS, double>(u0, args, err);
+        for (int v = 0; v < NV; ++v) u0[v] = d3::reg(u0planes[v * var_stride + i]);
+        double s = wave_speed<SYS, d3>(u0, args, err).v;
         if (s != s) {
             s = __longlong_as_double(0x7ff0000000000000ll);
             err |= ERR_NONFINITE;

@@ -15,6 +15,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "wcc_d3.cuh"
 #include "wcc_f2.cuh"
 
 namespace wcc {
@@ -475,8 +476,8 @@ __device__ __forceinline__ void limit_scalar(R (&e)[P + 1], R ubar, R vl, R vr, 
     } else {
         R wh0, wh1, wh2;
         if constexpr (P == 1) {
-            const R al = (R)args.alpha;
-            wh0 = pow((R)1 / (b0 + eps), al); wh1 = pow((R)1 / (b1 + eps), al); wh2 = pow((R)1 / (b2 + eps), al);
+            const double al = args.alpha;
+            wh0 = pow_any(recip(b0 + eps), al); wh1 = pow_any(recip(b1 + eps), al); wh2 = pow_any(recip(b2 + eps), al);
         } else {
             R up = e[0], um = e[0];
             sfor<1, P + 1>([&](auto Ki) {
@@ -488,12 +489,12 @@ __device__ __forceinline__ void limit_scalar(R (&e)[P + 1], R ubar, R vl, R vr, 
             const R sigma = fma(rr, rr, rl * rl);
             const R tp = (R)cfact(P) * e[P];
             const R st = sigma * (tp * tp);
-            const R al = (R)args.alpha;
-            wh0 = (R)1 + pow(st / fma(b0, b0, eps), al);
-            wh1 = pow(st / fma(b1, b1, eps), al);
-            wh2 = pow(st / fma(b2, b2, eps), al);
+            const double al = args.alpha;
+            wh0 = (R)1 + pow_any(div_any(st, fma(b0, b0, eps)), al);
+            wh1 = pow_any(div_any(st, fma(b1, b1, eps)), al);
+            wh2 = pow_any(div_any(st, fma(b2, b2, eps)), al);
         }
-        const R inv = (R)1 / (wh0 + wh1 + wh2);
+        const R inv = recip(wh0 + wh1 + wh2);
         w1 = wh1 * inv;
         w2 = wh2 * inv;
         w0 = (R)1 - (w1 + w2);
@@ -549,20 +550,19 @@ __device__ __forceinline__ bool euler_char(const R (&U)[3], R gamma, EulerChar<R
     const R g1 = gamma - (R)1;
     const R p = g1 * fma((R)-0.5 * U[1], u, U[2]);
     const R c2 = gamma * p * irho;
-    R ic;
-    if constexpr (f32) {
-        ic = rsqrt_approx(c2);  // the basis only needs FP32 accuracy
-        E.c = c2 * ic;
-    } else {
-        E.c = sqrt(c2);
-        ic = (R)1 / E.c;
-    }
     E.u = u;
     E.nu = -u;
     E.hu2 = (R)0.5 * u * u;
     E.H = (U[2] + p) * irho;
-    E.b1h = (R)0.5 * g1 * ic * ic;
-    E.ich = (R)0.5 * ic;
+    if constexpr (f32) {
+        const R ic = rsqrt_approx(c2);  // the basis only needs FP32 accuracy
+        E.c = c2 * ic;
+        E.b1h = (R)0.5 * g1 * ic * ic;
+        E.ich = (R)0.5 * ic;
+    } else {
+        E.c = sqrt_half_rsqrt(c2, E.ich);
+        E.b1h = (R)2 * g1 * (E.ich * E.ich);
+    }
     return all_pos(U[0]) && all_pos(p);
 }
 
@@ -587,11 +587,12 @@ __device__ __forceinline__ R wave_speed(const R* u0, const StepArgs& args, unsig
             const R c2 = gamma * p * irho;
             return fabs(u) + c2 * rsqrt_approx(c2);
         } else {
-            const R irho = (R)1 / rho;
+            const R irho = recip(rho);
             const R u = u0[1] * irho;
             const R p = g1 * fma((R)-0.5 * u0[1], u, u0[2]);
             if (!all_pos(rho) || !all_pos(p)) err |= ERR_POSITIVITY;
-            return fabs(u) + sqrt(gamma * p * irho);
+            R half_rsqrt;
+            return fabs(u) + sqrt_half_rsqrt(gamma * p * irho, half_rsqrt);
         }
     }
 }
