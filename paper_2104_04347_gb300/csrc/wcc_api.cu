@@ -237,6 +237,7 @@ StepArgs make_args(wcc_ctx* h, int cur, int parity, double cfl, double dt_fixed)
     a.limiter = h->opt.limiter;
     a.alpha_is_two = (h->opt.alpha == 2.0);
     a.dx = h->dx;
+    a.inv_dx = 1.0 / h->dx;
     a.cfl = cfl;
     a.cfl_mode = cfl > 0.0 ? 1 : 0;
     a.cfl_bits = (unsigned long long)__double_as_longlong_host(cfl);

@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(kThreadsMixed, (mixed_min_ctas<PA>() < mixed_m
         else
             mixed_tile2<SYS, PB, true, true>(io, ff_make(z.lam_hi, z.lam_lo), ph, rec, speed, err);
         reduce_and_finish<float, kThreadsMixed>(speed, err, z.dt, st, ntiles, b.hist + (long long)i * b.hist_cap, b.hist_cap,
-                                 b.parity, 1, b.phys.cfl, I.dx);
+                                 b.parity, 1, b.phys.cfl, I.dx, 0.0);
     }
 }
 

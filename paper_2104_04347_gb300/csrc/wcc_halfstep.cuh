@@ -38,13 +38,54 @@ __device__ __forceinline__ T warp_max(T v) {
     return v;
 }
 
+// Bit patterns of non-negative numbers, and the largest of a warp's.
+__device__ __forceinline__ unsigned speed_key(float s) { return __float_as_uint(s); }
+__device__ __forceinline__ unsigned long long speed_key(double s) {
+    return (unsigned long long)__double_as_longlong(s);
+}
+__device__ __forceinline__ unsigned warp_max_key(unsigned k) { return __reduce_max_sync(0xffffffffu, k); }
+__device__ __forceinline__ unsigned long long warp_max_key(unsigned long long k) {
+    const unsigned hi = (unsigned)(k >> 32);
+    const unsigned m = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned lo = __reduce_max_sync(0xffffffffu, hi == m ? (unsigned)k : 0u);
+    return ((unsigned long long)m << 32) | lo;
+}
+
+// dt = cfl dx / amax and lam = dt / dx of the next half-step.  FP64 kernels
+// take the quotients from a reciprocal with the remainder added back: the
+// bookkeeping is a serial chain at the end of a launch, where a warp's FP64
+// instruction takes 64 cycles and a division nine of them.  The FP32 kernels
+// keep the divisions (the other form costs them registers: two half-steps per
+// launch at P = 2 ran 1.3 % slower).
+template <bool F32>
+__device__ __forceinline__ void next_step(DevState* st, double cfl, double dx, double inv_dx, double amax) {
+    double dt, lam;
+    const double x = cfl * dx;
+    if (!F32 && mid_range(amax) && mid_range(x) && mid_range(inv_dx)) {
+        const d3 a(amax), n(x), ix(inv_dx);
+        const d3 r = recip(a), q = n * r;
+        const d3 t = fma(fma(-q, a, n), r, q);
+        const d3 l = t * ix;
+        dt = t.v;
+        lam = fma(fma(-l, d3(dx), t), ix, l).v;
+    } else {
+        dt = x / amax;
+        lam = dt / dx;
+    }
+    st->next_dt = dt;
+    st->next_lam = lam;
+    if (F32) split_to_floats(lam, st->next_lam_hi, st->next_lam_lo);
+    st->next_cfl = cfl;
+}
+
 // Bookkeeping of a solver state after the last CTA of a half-step finished:
 // publish the new stage's bound, clear the slots the next launches
 // accumulate into, record dt, advance t and prepare the next CFL step.
-// FP32 kernels (f32) accumulate the bound in amax_f32.
-__device__ __forceinline__ void finalize_state(DevState* st, bool f32, double dt, double* hist, long long hist_cap,
-                                               int parity, int cfl_mode, double cfl, double dx) {
-    if (f32) {
+// FP32 kernels (F32) accumulate the bound in amax_f32.
+template <bool F32>
+__device__ __forceinline__ void finalize_state(DevState* st, double dt, double* hist, long long hist_cap,
+                                               int parity, int cfl_mode, double cfl, double dx, double inv_dx) {
+    if (F32) {
         const float fm = __uint_as_float(st->amax_f32[parity ^ 1]);
         st->amax_bits[parity ^ 1] = (unsigned long long)__double_as_longlong((double)fm);
         st->amax_f32[parity] = 0u;
@@ -59,13 +100,7 @@ __device__ __forceinline__ void finalize_state(DevState* st, bool f32, double dt
     st->blocks_done = 0u;
     if (not_finite(dt)) st->err |= ERR_NONFINITE;
     if (cfl_mode) {
-        const double amax = __longlong_as_double((long long)st->amax_bits[parity ^ 1]);
-        const double ndt = cfl * dx / amax;
-        const double nlam = ndt / dx;
-        st->next_dt = ndt;
-        st->next_lam = nlam;
-        split_to_floats(nlam, st->next_lam_hi, st->next_lam_lo);
-        st->next_cfl = cfl;
+        next_step<F32>(st, cfl, dx, inv_dx, __longlong_as_double((long long)st->amax_bits[parity ^ 1]));
     } else {
         st->next_cfl = 0.0;
     }
@@ -78,51 +113,55 @@ __device__ __forceinline__ void finalize_state(DevState* st, bool f32, double dt
 template <class T, int NT = kThreads>
 __device__ __forceinline__ void reduce_and_finish(T speed, unsigned err, double dt, DevState* st, long long ctas,
                                                   double* hist, long long hist_cap, int parity, int cfl_mode,
-                                                  double cfl, double dx) {
+                                                  double cfl, double dx, double inv_dx) {
     // One block barrier: the warps' maxima and error bits meet in shared
     // memory, thread 0 combines them, posts them and counts the CTA; the CTA
     // that counts last finishes the launch's bookkeeping.  The barrier also
     // guarantees that every warp is done with the tile's shared records.
-    __shared__ T s_max[NT / 32];
+    using Key = decltype(speed_key(speed));
+    __shared__ Key s_max[NT / 32];
     __shared__ unsigned s_err[NT / 32];
     // NaN must win the max: map it to +Inf and flag it
     if (speed != speed) {
         speed = (T)INFINITY;
         err |= ERR_NONFINITE;
     }
-    speed = warp_max<T>(speed);
+    // (the bits of non-negative numbers order like the numbers: the maxima are
+    // taken on the integer pipe)
+    Key key = speed_key(speed);
+    key = warp_max_key(key);
     err = __reduce_or_sync(0xffffffffu, err);
     if ((threadIdx.x & 31) == 0) {
-        s_max[threadIdx.x >> 5] = speed;
+        s_max[threadIdx.x >> 5] = key;
         s_err[threadIdx.x >> 5] = err;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        T m = s_max[0];
+        Key m = s_max[0];
         unsigned e = s_err[0];
 #pragma unroll
         for (int w = 1; w < NT / 32; ++w) {
-            m = fmax(m, s_max[w]);
+            m = s_max[w] > m ? s_max[w] : m;
             e |= s_err[w];
         }
         if constexpr (sizeof(T) == 8) {
-            if (m > 0.0) atomicMax(&st->amax_bits[parity ^ 1], (unsigned long long)__double_as_longlong(m));
+            if (m) atomicMax(&st->amax_bits[parity ^ 1], m);
         } else {
-            if (m > 0.f) atomicMax(&st->amax_f32[parity ^ 1], __float_as_uint(m));
+            if (m) atomicMax(&st->amax_f32[parity ^ 1], m);
         }
         if (e) atomicOr(&st->err, e);
         __threadfence();
         const unsigned done = atomicAdd(&st->blocks_done, 1u);
         if (done == (unsigned)(ctas - 1)) {
             __threadfence();
-            finalize_state(st, sizeof(T) == 4, dt, hist, hist_cap, parity, cfl_mode, cfl, dx);
+            finalize_state<sizeof(T) == 4>(st, dt, hist, hist_cap, parity, cfl_mode, cfl, dx, inv_dx);
         }
     }
 }
 template <class T, int NT = kThreads>
 __device__ __forceinline__ void finish_halfstep(T speed, unsigned err, double dt, const StepArgs& args) {
     reduce_and_finish<T, NT>(speed, err, dt, args.st, (long long)gridDim.x, args.hist, args.hist_cap, args.parity,
-                             args.cfl_mode, args.cfl, args.dx);
+                             args.cfl_mode, args.cfl, args.dx, args.inv_dx);
 }
 
 template <int SYS, int P>
@@ -169,7 +208,7 @@ __global__ void __launch_bounds__(kThreads) halfstep_fp64(const StepArgs args) {
     double speed = 0.0;
     unsigned err = 0u;
     if (t < kTile && i < args.n_new) {
-        d3 e[NV][K], ubar[NV], vl[NV], vr[NV];
+        d3 e[NV][K], ubar[NV], dl[NV], dr[NV];
         sfor<0, NV>([&](auto V) {
             constexpr int v = decltype(V)::value;
             d3 vL[K], vR[K];
@@ -179,40 +218,50 @@ __global__ void __launch_bounds__(kThreads) halfstep_fp64(const StepArgs args) {
                 vR[k] = d3::reg(rec[2 * NV + v * K + k][t + 1]);
             });
             ubar[v] = d3::reg(rec[v][t]) + d3::reg(rec[NV + v][t + 1]);
-            vl[v] = vL[0];
-            vr[v] = vR[0];
-            derivatives_and_point_value<P, d3>(ubar[v], vL, vR, e[v]);
+            dl[v] = ubar[v] - vL[0];
+            dr[v] = vR[0] - ubar[v];
+            high_derivatives<P, d3>(vL, vR, e[v]);
         });
 
-        if (args.limiter) {
-            if constexpr (NV == 1) {
-                limit_scalar<P, d3>(e[0], ubar[0], vl[0], vr[0], args);
-            } else {
-                // Sec. 4: limit characteristic variables L(ubar) U, map back with R(ubar).
-                EulerChar<d3> E;
-                if (!euler_char<d3>(ubar, d3(args.gamma), E)) err |= ERR_POSITIVITY;
-                d3 ce[3][K], cub[3], cvl[3], cvr[3];
-                E.left(ubar[0], ubar[1], ubar[2], cub);
-                E.left(vl[0], vl[1], vl[2], cvl);
-                E.left(vr[0], vr[1], vr[2], cvr);
-                sfor<0, K>([&](auto Ki) {
-                    constexpr int k = decltype(Ki)::value;
-                    d3 w[3];
-                    E.left(e[0][k], e[1][k], e[2][k], w);
-                    ce[0][k] = w[0];
-                    ce[1][k] = w[1];
-                    ce[2][k] = w[2];
-                });
-                sfor<0, 3>([&](auto Ii) {
-                    constexpr int r = decltype(Ii)::value;
-                    limit_scalar<P, d3>(ce[r], cub[r], cvl[r], cvr[r], args);
-                });
-                sfor<0, K>([&](auto Ki) {
-                    constexpr int k = decltype(Ki)::value;
-                    E.right(ce[0][k], ce[1][k], ce[2][k], e[0][k], e[1][k], e[2][k]);
-                });
-            }
+        if (!args.limiter) {
+            sfor<0, NV>([&](auto V) {
+                constexpr int v = decltype(V)::value;
+                e[v][1] = first_derivative<P, d3>(e[v], dl[v], dr[v]);
+            });
+        } else if constexpr (NV == 1) {
+            e[0][1] = first_derivative<P, d3>(e[0], dl[0], dr[0]);
+            limit_deviation<P, d3>(e[0], dl[0], dr[0], args);
+        } else {
+            // Sec. 4: limit characteristic variables L(ubar) U, map back with
+            // R(ubar).  e_1 is linear in the differences and the higher
+            // coefficients, so it is formed after the projection.
+            EulerChar<d3> E;
+            if (!euler_char<d3>(ubar, d3(args.gamma), E)) err |= ERR_POSITIVITY;
+            d3 ce[3][K], cdl[3], cdr[3];
+            E.left(dl[0], dl[1], dl[2], cdl);
+            E.left(dr[0], dr[1], dr[2], cdr);
+            sfor<2, K>([&](auto Ki) {
+                constexpr int k = decltype(Ki)::value;
+                d3 w[3];
+                E.left(e[0][k], e[1][k], e[2][k], w);
+                ce[0][k] = w[0];
+                ce[1][k] = w[1];
+                ce[2][k] = w[2];
+            });
+            sfor<0, 3>([&](auto Ii) {
+                constexpr int r = decltype(Ii)::value;
+                ce[r][1] = first_derivative<P, d3>(ce[r], cdl[r], cdr[r]);
+                limit_deviation<P, d3>(ce[r], cdl[r], cdr[r], args);
+            });
+            sfor<1, K>([&](auto Ki) {
+                constexpr int k = decltype(Ki)::value;
+                E.right(ce[0][k], ce[1][k], ce[2][k], e[0][k], e[1][k], e[2][k]);
+            });
         }
+        sfor<0, NV>([&](auto V) {  // the limiter keeps the cell average
+            constexpr int v = decltype(V)::value;
+            e[v][0] = point_value<P, d3>(ubar[v], e[v]);
+        });
 
         bool bad = false;
         sfor<0, NV>([&](auto V) {

@@ -77,7 +77,7 @@ struct StepArgs {
     int bc;
     int limiter;
     int alpha_is_two;
-    double dx;
+    double dx, inv_dx;
     int cfl_mode;     // 1: dt from the CFL number (cfl > 0); 0: dt_fixed
     int pad_;
     unsigned long long cfl_bits;  // bit pattern of cfl (integer comparison, no FP64 pipe)
@@ -233,6 +233,13 @@ struct ParentRecord {
     R vtx[NV][P + 1];
 };
 
+// x times a constant, without the multiplication when it is 1
+template <bool ONE, class R>
+__device__ __forceinline__ R times(R x, double w) {
+    if constexpr (ONE) return x;
+    else return x * (R)w;
+}
+
 // Space-time Taylor table X[v][a][b] (a + b <= P) of one cell from its
 // Taylor coefficients c, and the flux coefficients F0[v][b] at a = 0.
 template <int SYS, int P, class R>
@@ -254,7 +261,7 @@ __device__ __forceinline__ void ck_table(const R (&c)[nvars(SYS)][P + 1], R lam,
             sfor<0, P - b>([&](auto Ai) {
                 constexpr int aa = decltype(Ai)::value;
                 constexpr double w = (aa + 1.0) / (b + 1.0);
-                X[0][aa][b + 1] = -(la * (R)w) * X[0][aa + 1][b];
+                X[0][aa][b + 1] = -times<w == 1.0>(la, w) * X[0][aa + 1][b];
             });
         });
         sfor<0, K>([&](auto Bi) {
@@ -288,7 +295,7 @@ __device__ __forceinline__ void ck_table(const R (&c)[nvars(SYS)][P + 1], R lam,
                 sfor<0, P - b>([&](auto Ai) {
                     constexpr int aa = decltype(Ai)::value;
                     constexpr double w = (aa + 1.0) / (b + 1.0);
-                    X[0][aa][b + 1] = -(lam * (R)w) * F[aa + 1][b];
+                    X[0][aa][b + 1] = -times<w == 1.0>(lam, w) * F[aa + 1][b];
                 });
             }
             F0[0][b] = F[0][b];
@@ -337,7 +344,7 @@ __device__ __forceinline__ void ck_table(const R (&c)[nvars(SYS)][P + 1], R lam,
                 sfor<0, P - b>([&](auto Ai) {
                     constexpr int aa = decltype(Ai)::value;
                     constexpr double wgt = (aa + 1.0) / (b + 1.0);
-                    const R lw = lam * (R)wgt;
+                    const R lw = times<wgt == 1.0>(lam, wgt);
                     X[0][aa][b + 1] = -lw * X[1][aa + 1][b];
                     X[1][aa][b + 1] = -lw * Fm[aa + 1][b];
                     X[2][aa][b + 1] = -lw * FE[aa + 1][b];
@@ -367,16 +374,19 @@ __device__ __forceinline__ void parent_record(const R (&c)[nvars(SYS)][P + 1], R
             constexpr int b = decltype(Bi)::value;
             fbar = fma((R)(1.0 / (b + 1.0)), F0[v][b], fbar);
         });
-        // Eqs. SubEq:1DCellAVGR / SubEq:1DCellAVGL: half-cell averages.
-        R ur = c[v][0], ul = c[v][0];
-        sfor<1, K>([&](auto Ki) {
+        // Eqs. SubEq:1DCellAVGR / SubEq:1DCellAVGL: the half-cell averages
+        // share their even part, and the flux joins the odd one:
+        // A, B = even / 2 +- (odd / 2 + lam fbar).
+        R even = (R)0.5 * c[v][0], odd = (R)0.125 * c[v][1];
+        sfor<2, K>([&](auto Ki) {
             constexpr int k = decltype(Ki)::value;
-            constexpr double wk = 1.0 / ((k + 1.0) * cpow2(k));
-            ur = fma((R)wk, c[v][k], ur);
-            ul = fma((R)((k & 1) ? -wk : wk), c[v][k], ul);
+            constexpr double wk = 0.5 / ((k + 1.0) * cpow2(k));
+            if constexpr (k & 1) odd = fma((R)wk, c[v][k], odd);
+            else even = fma((R)wk, c[v][k], even);
         });
-        out.A[v] = fma(lam, fbar, (R)0.5 * ur);
-        out.B[v] = fma(-lam, fbar, (R)0.5 * ul);
+        const R g = fma(lam, fbar, odd);
+        out.A[v] = even + g;
+        out.B[v] = even - g;
         // Eq. SubEq:Cal_1D_Derivatives_4: vertex values at t^{n+1/2}.
         sfor<0, K>([&](auto Ki) {
             constexpr int k = decltype(Ki)::value;
@@ -416,80 +426,113 @@ __device__ __forceinline__ void derivatives_and_point_value(R ubar, const R (&vL
     e[0] = u0;
 }
 
-// WENO-type limiter of Sec. 2.2 on one scalar (or characteristic) component.
-// e: Taylor coefficients of u_0 (overwritten by u_*), ubar its cell average,
-// vl / vr the time-extrapolated vertex values u_{i-1/2}, u_{i+1/2}.
+// Coefficients e_2 .. e_P of a new cell (Eq. SubEq:Cal_1D_Derivatives_3).
 template <int P, class R>
-__device__ __forceinline__ void limit_scalar(R (&e)[P + 1], R ubar, R vl, R vr, const StepArgs& args) {
-    const R s1 = (R)2 * (ubar - vl);   // Eq. SubEq:1DU12, slope of u_1
-    const R s2 = (R)2 * (vr - ubar);   // slope of u_2
+__device__ __forceinline__ void high_derivatives(const R (&vL)[P + 1], const R (&vR)[P + 1], R (&e)[P + 1]) {
+    sfor<0, P - 1>([&](auto Ii) {
+        constexpr int k = P - 1 - decltype(Ii)::value;  // P - 1 .. 1
+        R s = vR[k] - vL[k];
+        sfor<3, P - k + 1>([&](auto Mi) {
+            constexpr int m = decltype(Mi)::value;
+            if constexpr (m & 1) {
+                constexpr double cm = 2.0 * cbinom(k + m, m) * cpow2(-m);
+                s = fma((R)-cm, e[k + m], s);
+            }
+        });
+        e[k + 1] = s * (R)(1.0 / (k + 1.0));
+    });
+}
+
+// e_1 of the same equation from the one-sided differences dl = ubar - u_{i-1/2}
+// and dr = u_{i+1/2} - ubar: u_{i+1/2} - u_{i-1/2} less the odd terms above.
+template <int P, class R>
+__device__ __forceinline__ R first_derivative(const R (&e)[P + 1], R dl, R dr) {
+    R s = dl + dr;
+    sfor<3, P + 1>([&](auto Mi) {
+        constexpr int m = decltype(Mi)::value;
+        if constexpr (m & 1) s = fma((R)(-2.0 * cpow2(-m)), e[m], s);
+    });
+    return s;
+}
+
+// Point value less the cell average: -sum over even k >= 2 of e_k / ((k+1) 2^k)
+// (Eq. 1DCalU).
+template <int P, class R>
+__device__ __forceinline__ R point_value(R ubar, const R (&e)[P + 1]) {
+    R u0 = ubar;
+    sfor<2, P + 1>([&](auto Ki) {
+        constexpr int k = decltype(Ki)::value;
+        if constexpr ((k & 1) == 0) u0 = fma((R)(-1.0 / ((k + 1.0) * cpow2(k))), e[k], u0);
+    });
+    return u0;
+}
+
+// WENO-type limiter of Sec. 2.2 on one scalar (or characteristic) component
+// in deviation form: e[1..P] the Taylor coefficients of u_0 (overwritten by
+// those of u_*), dl = ubar - u_{i-1/2}, dr = u_{i+1/2} - ubar with the
+// time-extrapolated vertex values.  The limiter keeps the cell average, and
+// nothing in it depends on it.  The two residuals of sigma are the same
+// number: the unlimited polynomial's difference between its ends is
+// u_{i+1/2} - u_{i-1/2} by construction of e_1, so both equal
+//   r = (even part at the ends less the average) + (dl - dr) / 2.
+template <int P, class R>
+__device__ __forceinline__ void limit_deviation(R (&e)[P + 1], R dl, R dr, const StepArgs& args) {
+    const R s1 = dl + dl;  // Eq. SubEq:1DU12, slope of u_1
+    const R s2 = dr + dr;  // slope of u_2
     // beta_0 (Eq. 1DSmoothIndicator) as a quadratic form in e_1..e_P
-    R b0 = (R)0;
+    R b0;
     sfor<1, P + 1>([&](auto Ji) {
         constexpr int j = decltype(Ji)::value;
-        R row = (R)0;
-        sfor<j, P + 1>([&](auto Li) {
+        R row = times<csmooth(j, j) == 1.0>(e[j], csmooth(j, j));
+        sfor<j + 1, P + 1>([&](auto Li) {
             constexpr int l = decltype(Li)::value;
-            constexpr double cjl = (l == j ? 1.0 : 2.0) * csmooth(j, l);
+            constexpr double cjl = 2.0 * csmooth(j, l);
             if constexpr (cjl != 0.0) row = fma((R)cjl, e[l], row);
         });
-        b0 = fma(row, e[j], b0);
+        if constexpr (j == 1) b0 = row * e[1];
+        else b0 = fma(row, e[j], b0);
     });
     const R b1 = s1 * s1, b2 = s2 * s2;
     const R eps = (R)args.eps;
+    R st;  // sigma tau
+    if constexpr (P >= 2) {
+        R r = (R)0.5 * (dl - dr);
+        sfor<2, P + 1>([&](auto Ki) {
+            constexpr int k = decltype(Ki)::value;
+            if constexpr ((k & 1) == 0) r = fma((R)(cpow2(-k) * k / (k + 1.0)), e[k], r);
+        });
+        const R y = e[P] * r;
+        st = ((R)(2.0 * cfact(P) * cfact(P)) * y) * y;
+    }
     R w0, w1, w2;
     if (args.alpha_is_two) {
         // Multiplied through by the denominators, so that one reciprocal
         // normalises the weights; w0 = 1 - w1 - w2 is exactly 1 when the
         // other two vanish.
-        R h0, h1, h2;
         if constexpr (P == 1) {
             // Eq. 1D2ndOrderWeights: w_m ~ (beta_m + eps)^-2
             const R d0 = b0 + eps, d1 = b1 + eps, d2 = b2 + eps;
             const R p12 = d1 * d2, p02 = d0 * d2, p01 = d0 * d1;
-            h0 = p12 * p12;
-            h1 = p02 * p02;
-            h2 = p01 * p01;
+            const R inv = recip(fma(p12, p12, fma(p02, p02, p01 * p01)));
+            w1 = (p02 * inv) * p02;
+            w2 = (p01 * inv) * p01;
         } else {
             // Eq. 1DHighOrderWeights: w0 ~ 1 + (st/d0)^2, w_m ~ (st/d_m)^2
-            R up = e[0], um = e[0];
-            sfor<1, P + 1>([&](auto Ki) {
-                constexpr int k = decltype(Ki)::value;
-                up = fma((R)chalf(k, false), e[k], up);
-                um = fma((R)chalf(k, true), e[k], um);
-            });
-            const R rr = up - vr, rl = um - vl;
-            const R sigma = fma(rr, rr, rl * rl);
-            const R tp = (R)cfact(P) * e[P];
-            const R st = sigma * (tp * tp);
             const R d0 = fma(b0, b0, eps), d1 = fma(b1, b1, eps), d2 = fma(b2, b2, eps);
-            const R p12 = d1 * d2, p02 = d0 * d2, p01 = d0 * d1;
-            const R s12 = st * p12, s02 = st * p02, s01 = st * p01;
-            h0 = fma(d0 * p12, d0 * p12, s12 * s12);
-            h1 = s02 * s02;
-            h2 = s01 * s01;
+            const R p12 = d1 * d2, sd0 = st * d0;
+            const R s12 = st * p12, s02 = sd0 * d2, s01 = sd0 * d1, p = d0 * p12;
+            const R inv = recip(fma(p, p, fma(s12, s12, fma(s02, s02, s01 * s01))));
+            w1 = (s02 * inv) * s02;
+            w2 = (s01 * inv) * s01;
         }
-        const R inv = recip(h0 + h1 + h2);
-        w1 = h1 * inv;
-        w2 = h2 * inv;
-        w0 = (R)1 - (w1 + w2);
     } else {
+        const double al = args.alpha;
         R wh0, wh1, wh2;
         if constexpr (P == 1) {
-            const double al = args.alpha;
-            wh0 = pow_any(recip(b0 + eps), al); wh1 = pow_any(recip(b1 + eps), al); wh2 = pow_any(recip(b2 + eps), al);
+            wh0 = pow_any(recip(b0 + eps), al);
+            wh1 = pow_any(recip(b1 + eps), al);
+            wh2 = pow_any(recip(b2 + eps), al);
         } else {
-            R up = e[0], um = e[0];
-            sfor<1, P + 1>([&](auto Ki) {
-                constexpr int k = decltype(Ki)::value;
-                up = fma((R)chalf(k, false), e[k], up);
-                um = fma((R)chalf(k, true), e[k], um);
-            });
-            const R rr = up - vr, rl = um - vl;
-            const R sigma = fma(rr, rr, rl * rl);
-            const R tp = (R)cfact(P) * e[P];
-            const R st = sigma * (tp * tp);
-            const double al = args.alpha;
             wh0 = (R)1 + pow_any(div_any(st, fma(b0, b0, eps)), al);
             wh1 = pow_any(div_any(st, fma(b1, b1, eps)), al);
             wh2 = pow_any(div_any(st, fma(b2, b2, eps)), al);
@@ -497,10 +540,9 @@ __device__ __forceinline__ void limit_scalar(R (&e)[P + 1], R ubar, R vl, R vr, 
         const R inv = recip(wh0 + wh1 + wh2);
         w1 = wh1 * inv;
         w2 = wh2 * inv;
-        w0 = (R)1 - (w1 + w2);
     }
+    w0 = (R)1 - (w1 + w2);
     // Eq. 1DLimitedPolynomial, coefficient by coefficient.
-    e[0] = fma(w0, e[0], (w1 + w2) * ubar);
     e[1] = fma(w0, e[1], fma(w1, s1, w2 * s2));
     sfor<2, P + 1>([&](auto Ki) { e[decltype(Ki)::value] *= w0; });
 }
@@ -548,11 +590,12 @@ __device__ __forceinline__ bool euler_char(const R (&U)[3], R gamma, EulerChar<R
     const R irho = recip(U[0]);
     const R u = U[1] * irho;
     const R g1 = gamma - (R)1;
-    const R p = g1 * fma((R)-0.5 * U[1], u, U[2]);
+    const R hu = (R)0.5 * u;
+    const R p = g1 * fma(-hu, U[1], U[2]);
     const R c2 = gamma * p * irho;
     E.u = u;
     E.nu = -u;
-    E.hu2 = (R)0.5 * u * u;
+    E.hu2 = hu * u;
     E.H = (U[2] + p) * irho;
     if constexpr (f32) {
         const R ic = rsqrt_approx(c2);  // the basis only needs FP32 accuracy

@@ -144,6 +144,7 @@ extern "C" int wcc_advance_static(int system, int P, int bc, int64_t N, const do
     a.limiter = o.limiter;
     a.alpha_is_two = (o.alpha == 2.0);
     a.dx = (domain[1] - domain[0]) / (double)N;
+    a.inv_dx = 1.0 / a.dx;
     a.cfl = cfl;
     a.cfl_mode = 1;
     a.cfl_bits = (unsigned long long)__double_as_longlong_host(cfl);
