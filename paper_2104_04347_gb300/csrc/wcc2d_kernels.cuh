@@ -19,6 +19,7 @@
 #include <algorithm>
 
 #include "wcc2d_scheme.cuh"
+#include "wcc_pdl.cuh"
 
 namespace wcc2d {
 
@@ -168,6 +169,7 @@ __global__ void __launch_bounds__(TW, min_ctas2d<T>()) halfstep2d(const Step2D a
     const int j0 = blockIdx.y * a.rows_per_cta;
     const int rows = min(a.rows_per_cta, a.ny_new - j0);
 
+    wcc::pdl_begin();
     const double dt = step_dt2d(a);
     const T lamx = (T)(dt * a.inv_dx), lamy = (T)(dt * a.inv_dy);
     const T idx = (T)a.inv_dx, idy = (T)a.inv_dy;
@@ -365,8 +367,7 @@ cudaError_t launch_strips2d(const Step2D& a, cudaStream_t stream) {
     static_assert(smem <= 48 * 1024 - 256, "the shared ring and the static shared words must fit without the opt-in attribute");
     if (a.resident) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(a.resident, halfstep2d<SYS, P, T, TW>, TW, smem);
     const dim3 grid((a.nx_new + TW - 2) / (TW - 1), (a.ny_new + a.rows_per_cta - 1) / a.rows_per_cta);
-    halfstep2d<SYS, P, T, TW><<<grid, TW, smem, stream>>>(a);
-    return cudaGetLastError();
+    return wcc::launch_pdl<Step2D>(halfstep2d<SYS, P, T, TW>, grid, TW, smem, stream, a);
 }
 
 // Launch one half-step of system SYS at degree P in type T.
@@ -475,6 +476,7 @@ __global__ void __launch_bounds__(TW, 4) halfstep2d_mx(const Step2D a) {
     const int j0 = blockIdx.y * a.rows_per_cta;
     const int rows = min(a.rows_per_cta, a.ny_new - j0);
 
+    wcc::pdl_begin();
     const double dt = step_dt2d(a);
     // lam rounded to float in every term, the leading flux terms included:
     // the half-step is one of size fl(lam) dx, the same in all its Taylor
@@ -695,8 +697,7 @@ cudaError_t launch_halfstep2d_mx_t(const Step2D& a, cudaStream_t stream) {
     static_assert(smem <= 48 * 1024 - 256, "the shared ring and the static shared words must fit without the opt-in attribute");
     if (a.resident) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(a.resident, halfstep2d_mx<SYS, P, TW>, TW, smem);
     const dim3 grid((a.nx_new + TW - 2) / (TW - 1), (a.ny_new + a.rows_per_cta - 1) / a.rows_per_cta);
-    halfstep2d_mx<SYS, P, TW><<<grid, TW, smem, stream>>>(a);
-    return cudaGetLastError();
+    return wcc::launch_pdl<Step2D>(halfstep2d_mx<SYS, P, TW>, grid, TW, smem, stream, a);
 }
 
 }  // namespace wcc2d

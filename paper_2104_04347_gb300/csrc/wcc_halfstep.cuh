@@ -16,6 +16,7 @@
 //      device without a host round trip.
 #pragma once
 
+#include "wcc_pdl.cuh"
 #include "wcc_scheme.cuh"
 
 namespace wcc {
@@ -174,6 +175,7 @@ __global__ void __launch_bounds__(kThreads) halfstep_fp64(const StepArgs args) {
     const int t = threadIdx.x;
     const long long first_new = (long long)blockIdx.x * kTile;
 
+    pdl_begin();
     const StepSize z = step_size(args);
     const double dt = z.dt;
     const double lam = z.lam;
@@ -186,7 +188,7 @@ __global__ void __launch_bounds__(kThreads) halfstep_fp64(const StepArgs args) {
             constexpr int v = decltype(V)::value;
             sfor<0, K>([&](auto Ki) {
                 constexpr int k = decltype(Ki)::value;
-                c[v][k] = d3::reg(__ldg(args.in64 + (long long)(v * K + k) * args.pitch + p));
+                c[v][k] = d3::reg(args.in64[(long long)(v * K + k) * args.pitch + p]);
             });
         });
         ParentRecord<SYS, P, d3> r;

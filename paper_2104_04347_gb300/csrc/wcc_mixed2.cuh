@@ -366,12 +366,12 @@ __device__ __forceinline__ void mixed_load_parents(const TileIO& io, ff2 (&ub)[n
         constexpr int v = decltype(V)::value;
         const float* p0 = io.in32 + (long long)(v * NP + 0) * io.pitch;
         const float* p1 = io.in32 + (long long)(v * NP + 1) * io.pitch;
-        ub[v].hi = f2(__ldg(p0 + pa), __ldg(p0 + pb));
-        ub[v].lo = COMP ? f2(__ldg(p1 + pa), __ldg(p1 + pb)) : f2(0.f);
+        ub[v].hi = f2(p0[pa], p0[pb]);
+        ub[v].lo = COMP ? f2(p1[pa], p1[pb]) : f2(0.f);
         sfor<1, K>([&](auto Ki) {
             constexpr int k = decltype(Ki)::value;
             const float* pk = io.in32 + (long long)(v * NP + k + 1) * io.pitch;
-            c[v][k] = f2(__ldg(pk + pa), __ldg(pk + pb));
+            c[v][k] = f2(pk[pa], pk[pb]);
         });
     });
 }
@@ -472,8 +472,8 @@ __device__ __forceinline__ void mixed_parent_records(const ff2 (&ub_in)[nvars(SY
         const ff2 Ac = A::half_plus(ub, lf, h);
         put(v, 2, Ac.hi);
         if constexpr (COMP) put(v, 3, Ac.lo);
-        f2 vt0(0.f);
-        sfor<1, K>([&](auto Mi) { vt0 += X[v][0][decltype(Mi)::value]; });
+        f2 vt0 = X[v][0][1];
+        sfor<2, K>([&](auto Mi) { vt0 += X[v][0][decltype(Mi)::value]; });
         put(v, 4, vt0 - average_minus_centre<P>(c[v]));
         sfor<1, K>([&](auto Ki) {
             constexpr int k = decltype(Ki)::value;
@@ -619,18 +619,22 @@ __device__ __forceinline__ float mixed_store(const TileIO& io, const ff2 (&ubn)[
 // io.first_new + c for c = 0..kTileMixed - 1.  rec: mixed2_smem_float2 float2
 // of shared memory.  Returns the larger of the thread's two cell speeds
 // (cells outside the stage count as 0) and error bits; the caller
-// synchronises the block before rec is written again.
-template <int SYS, int P, bool COMP, bool PARK = (P >= 3)>
-__device__ __forceinline__ void mixed_tile2(const TileIO& io, const ff lam, const StepArgs& args, float2* rec,
+// synchronises the block before rec is written again.  step() gives the
+// half-step's size; it is called after the parents' loads have been issued,
+// so that reading the device state does not delay them (the state's fields
+// decide a branch, which waits for them).
+template <int SYS, int P, bool COMP, bool PARK = (P >= 3), class Step>
+__device__ __forceinline__ void mixed_tile2(const TileIO& io, Step&& step, const StepArgs& args, float2* rec,
                                             float& speed, unsigned& err) {
     constexpr int NV = nvars(SYS);
     constexpr int K = P + 1;
     const int t = threadIdx.x;
-    const ff2 lam2{f2(lam.hi), f2(COMP ? lam.lo : 0.f)};
     {
         ff2 ub[NV];
         f2 c[NV][K];
         mixed_load_parents<SYS, P, COMP>(io, ub, c);
+        const StepSize& z = step();
+        const ff2 lam2{f2(z.lam_hi), f2(COMP ? z.lam_lo : 0.f)};
         mixed_parent_records<SYS, P, COMP, PARK>(ub, c, lam2, args, rec);
     }
     __syncthreads();
@@ -648,13 +652,14 @@ __device__ __forceinline__ void mixed_tile2(const TileIO& io, const ff lam, cons
 template <int SYS, int P, bool COMP = true, int TPC = mixed_tiles_per_cta<P>()>
 __global__ void __launch_bounds__(kThreadsMixed, mixed_min_ctas<P>()) halfstep_mixed2(const StepArgs args) {
     __shared__ float2 rec[mixed2_smem_float2<SYS, P>()];
-    const StepSize z = step_size(args);
+    pdl_begin();
+    StepSize z;
     float speed = 0.f;
     unsigned err = 0u;
     if constexpr (TPC == 1) {
         const TileIO io{args.in32, args.out32, args.pitch, args.n_old, args.n_new,
                         (long long)blockIdx.x * kTileMixed, args.parity, args.bc};
-        mixed_tile2<SYS, P, COMP>(io, ff_make(z.lam_hi, z.lam_lo), args, rec, speed, err);
+        mixed_tile2<SYS, P, COMP>(io, [&]() -> const StepSize& { return z = step_size(args); }, args, rec, speed, err);
     } else {
         const long long ntiles = (args.n_new + kTileMixed - 1) / kTileMixed;
         for (int r = 0; r < TPC; ++r) {
@@ -664,7 +669,8 @@ __global__ void __launch_bounds__(kThreadsMixed, mixed_min_ctas<P>()) halfstep_m
             const TileIO io{args.in32, args.out32, args.pitch, args.n_old, args.n_new,
                             tile * kTileMixed, args.parity, args.bc};
             float sp = 0.f;
-            mixed_tile2<SYS, P, COMP>(io, ff_make(z.lam_hi, z.lam_lo), args, rec, sp, err);
+            mixed_tile2<SYS, P, COMP>(
+                io, [&]() -> const StepSize& { return r ? z : (z = step_size(args)); }, args, rec, sp, err);
             speed = fmaxf(speed, sp);
         }
     }
@@ -802,7 +808,7 @@ struct PairIO {
 };
 
 // One tile of two staggered half-steps (temporal blocking, FP32 variants):
-// stage n (parity p) -> n + 1/2 -> n + 1 (parity p), both with the step lam2.
+// stage n (parity p) -> n + 1/2 -> n + 1 (parity p), both with the size step().
 // The tile owns final cells f0 .. f0 + kTileTB - 1; it loads the parents
 // o0 = f0 - 1 .. o0 + 2 kThreadsMixed - 1, builds the intermediate cells
 // m0 = o0 + p .. m0 + 2 kThreadsMixed - 2 in registers (each thread's two
@@ -814,8 +820,8 @@ struct PairIO {
 // parents.  Returns the largest speeds of the thread's intermediate and final
 // cells (cells outside the stages count as 0) and error bits; synchronises
 // the block, and the caller synchronises it again before rec is written.
-template <int SYS, int P, bool COMP, bool PARK = (P >= 3)>
-__device__ __forceinline__ void mixed_pair_tile(const PairIO& io, const ff2 lam2, const StepArgs& args, float2* rec,
+template <int SYS, int P, bool COMP, bool PARK = (P >= 3), class Step>
+__device__ __forceinline__ void mixed_pair_tile(const PairIO& io, Step&& step, const StepArgs& args, float2* rec,
                                                 float& mid_speed, float& fin_speed, unsigned& err) {
     constexpr int NV = nvars(SYS);
     constexpr int K = P + 1;
@@ -825,11 +831,13 @@ __device__ __forceinline__ void mixed_pair_tile(const PairIO& io, const ff2 lam2
     const long long o0 = f0 - 1;
     const long long m0 = o0 + p;
 
-    ff2 ub[NV];
+    ff2 ub[NV], lam2;
     f2 c[NV][K];
     {
         const TileIO io1{io.in32, nullptr, io.pitch, io.n_old, io.n_mid, m0, p, io.bc};
         mixed_load_parents<SYS, P, COMP>(io1, ub, c);
+        const StepSize& z = step();
+        lam2 = ff2{f2(z.lam_hi), f2(COMP ? z.lam_lo : 0.f)};
         mixed_parent_records<SYS, P, COMP, PARK>(ub, c, lam2, args, rec);
     }
     __syncthreads();
@@ -914,14 +922,14 @@ __device__ __forceinline__ void mixed_pair_tile(const PairIO& io, const ff2 lam2
 template <int SYS, int P, bool COMP = true>
 __global__ void __launch_bounds__(kThreadsMixed, mixed_min_ctas<P>()) halfstep_mixed2_tb2(const StepArgs args) {
     __shared__ float2 rec[mixed2_smem_float2<SYS, P>()];
+    pdl_begin();
     if (args.st->err & ERR_CFL) return;  // an earlier pair was refused: the caller steps singly from there
-    const StepSize z = step_size(args);
-    const ff2 lam2{f2(z.lam_hi), f2(COMP ? z.lam_lo : 0.f)};
+    StepSize z;
     const PairIO io{args.in32, args.out32, args.pitch, args.n_old, args.n_mid, args.n_new,
                     (long long)blockIdx.x * kTileTB, args.parity, args.bc};
     float mid = 0.f, fin = 0.f;
     unsigned err = 0u;
-    mixed_pair_tile<SYS, P, COMP>(io, lam2, args, rec, mid, fin, err);
+    mixed_pair_tile<SYS, P, COMP>(io, [&]() -> const StepSize& { return z = step_size(args); }, args, rec, mid, fin, err);
     const PairBook bk{args.st, args.hist, args.hist_cap, (long long)gridDim.x, args.dx, args.cfl, args.tb_nu_max,
                       args.cfl_mode, args.parity, nullptr, nullptr};
     finish_pair(mid, fin, err, z.dt, bk);

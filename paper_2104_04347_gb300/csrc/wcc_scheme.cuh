@@ -496,11 +496,12 @@ __device__ __forceinline__ void limit_deviation(R (&e)[P + 1], R dl, R dr, const
     const R eps = (R)args.eps;
     R st;  // sigma tau
     if constexpr (P >= 2) {
-        R r = (R)0.5 * (dl - dr);
-        sfor<2, P + 1>([&](auto Ki) {
+        R r = (R)(1.0 / 6.0) * e[2];
+        sfor<4, P + 1>([&](auto Ki) {
             constexpr int k = decltype(Ki)::value;
             if constexpr ((k & 1) == 0) r = fma((R)(cpow2(-k) * k / (k + 1.0)), e[k], r);
         });
+        r = fma((R)0.5, dl - dr, r);
         const R y = e[P] * r;
         st = ((R)(2.0 * cfact(P) * cfact(P)) * y) * y;
     }
