@@ -213,7 +213,7 @@ int wcc_launch_count(wcc_handle h, int64_t* launches);
 
 /* ------------------------------------------------------------------ batches
  * Many independent problems of one conservation law, advanced together: one
- * persistent kernel launch per half-step walks the tiles of every instance
+ * kernel launch per half-step covers the tiles of every instance
  * (cells are flattened across instances, so instances of very different N
  * share the GPU evenly).  Each instance keeps its own N, P, domain, boundary,
  * time and dt = cfl * dx_i / a_max,i (the scheme of Sec. 2 applied to each
@@ -250,7 +250,8 @@ int wcc_batch_get_times(wcc_batch b, double* t, int64_t count);
 int wcc_batch_get_state(wcc_batch b, int64_t* half_steps, int* parity);
 /* Half-step sizes of one instance (user index), as wcc_get_dt_history. */
 int wcc_batch_get_dt_history(wcc_batch b, int64_t instance, double* dts, int64_t cap, int64_t* n);
-/* Persistent grid of the step kernel in CTAs (0: all resident CTAs). */
+/* Grid of the step kernel in CTAs (0, the default: one CTA per tile; fewer
+ * CTAs walk the list of tiles). */
 int wcc_batch_set_grid(wcc_batch b, int ctas);
 /* Time the candidate grids (1..max resident CTAs per SM, and one CTA per
  * tile), each with one half-step per launch and, where the degree mix has
@@ -261,7 +262,7 @@ int wcc_batch_set_grid(wcc_batch b, int ctas);
  * wcc_batch_get_tuning reports both.  Allocates a temporary copy of the
  * current stage.  Synchronous. */
 int wcc_batch_autotune(wcc_batch b, double cfl, int* ctas);
-/* The launch configuration in use: *ctas the persistent grid of the step
+/* The launch configuration in use: *ctas the grid of the step
  * kernel, *tb_depth half-steps per launch (1 or 2).  Either may be NULL. */
 int wcc_batch_get_tuning(wcc_batch b, int* ctas, int* tb_depth);
 /* Two-half-step launches of a batch: *pairs taken, *fallbacks refused (a

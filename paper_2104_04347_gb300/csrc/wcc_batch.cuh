@@ -49,7 +49,7 @@ struct BatchArgs {
 };
 
 
-template <int SYS, int PA, int PB>
+template <int SYS, int PA, int PB, bool LOOP>
 __global__ void __launch_bounds__(kThreadsMixed, (mixed_min_ctas<PA>() < mixed_min_ctas<PB>() ? mixed_min_ctas<PA>()
                                                                                             : mixed_min_ctas<PB>()))
     batch_mixed(const BatchArgs b) {
@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(kThreadsMixed, (mixed_min_ctas<PA>() < mixed_m
     constexpr int SB = mixed2_smem_float2<SYS, PB>();
     __shared__ float2 rec[SA > SB ? SA : SB];
     pdl_begin();
-    for (long long tile = blockIdx.x; tile < b.total_tiles; tile += gridDim.x) {
+    for (long long tile = blockIdx.x; tile < b.total_tiles; tile += LOOP ? (long long)gridDim.x : b.total_tiles) {
         const int i = __ldg(b.tile_inst + tile);
         const BatchInstance& I = b.inst[i];
         DevState* st = b.st + i;
@@ -87,9 +87,8 @@ __global__ void __launch_bounds__(kThreadsMixed, (mixed_min_ctas<PA>() < mixed_m
 // first keeping the instance's state in tb_backup.  If any instance refuses
 // its pair, the batch's flag is set and the caller restores every instance
 // from tb_backup (the launch did not overwrite the input stages) and takes
-// that pair as two single half-steps; launches that find the flag set do
-// nothing.
-template <int SYS, int PA, int PB>
+// that pair as two single half-steps; launches after it do nothing.
+template <int SYS, int PA, int PB, bool LOOP>
 __global__ void __launch_bounds__(kThreadsMixed, (mixed_min_ctas<PA>() < mixed_min_ctas<PB>() ? mixed_min_ctas<PA>()
                                                                                             : mixed_min_ctas<PB>()))
     batch_mixed_tb2(const BatchArgs b) {
@@ -97,11 +96,14 @@ __global__ void __launch_bounds__(kThreadsMixed, (mixed_min_ctas<PA>() < mixed_m
     constexpr int SB = mixed2_smem_float2<SYS, PB>();
     __shared__ float2 rec[SA > SB ? SA : SB];
     pdl_begin();
-    if (*(volatile unsigned*)b.tb_refused) return;
-    for (long long tile = blockIdx.x; tile < b.total_tiles; tile += gridDim.x) {
+    const unsigned refused = *(volatile unsigned*)b.tb_refused;
+    for (long long tile = blockIdx.x; tile < b.total_tiles; tile += LOOP ? (long long)gridDim.x : b.total_tiles) {
         const int i = __ldg(b.tile_inst + tile);
         const BatchInstance& I = b.inst[i];
         DevState* st = b.st + i;
+        // a launch after the refusing one; the refusing launch itself, some of
+        // whose CTAs start after the flag is set, is completed
+        if (refused && (refused != pair_mark(st->step) || (st->err & ERR_CFL))) continue;
         const long long first = __ldg(b.tile_start + i);
         const long long ntiles = __ldg(b.tile_start + i + 1) - first;
         StepSize z;
@@ -187,22 +189,37 @@ __device__ __forceinline__ void convert_cell(double* q, float* pl, long long pit
     }
 }
 
+// Reading back, the tile's host-layout side (one run of doubles) goes through
+// shared memory so that consecutive threads write consecutive words: 96 M values
+// take 0.45 ms instead of 0.87 ms with a thread writing its cell's words one by
+// one.  Loading, the cache holds a cell's words between the thread's reads,
+// and the same detour was slower (0.37 against 0.30 ms).
 template <int SYS, int PA, int PB>
 __global__ void __launch_bounds__(kThreads) batch_convert(const BatchArgs b, double* aos, int to_planes) {
+    constexpr int NV = nvars(SYS);
+    __shared__ unsigned long long sm[kTile * NV * (PB + 1)];
     for (long long tile = blockIdx.x; tile < b.total_tiles; tile += gridDim.x) {
         const int i = __ldg(b.tile_inst + tile);
-        const BatchInstance I = b.inst[i];
-        const long long c = (tile - b.tile_start[i]) * kTile + threadIdx.x;
-        if (threadIdx.x >= kTile || c >= I.cells[b.parity]) continue;
-        const int P = I.group == 0 ? PA : PB;
-        const int K = P + 1, NV = nvars(SYS);
+        const BatchInstance& I = b.inst[i];
+        const long long c0 = (tile - b.tile_start[i]) * kTile;
+        const long long rest = I.cells[b.parity] - c0;
+        const int cnt = rest < kTile ? (int)rest : kTile;
+        const int row = NV * ((I.group == 0 ? PA : PB) + 1);
         float* pl = (to_planes ? b.out[I.group] : const_cast<float*>(b.in[I.group])) + I.offset;
         const long long pitch = b.pitch[I.group];
-        double* q0 = aos + I.aos_offset[b.parity] + c * NV * K;
-        if (I.group == 0)
-            convert_cell<PA + 1>(q0, pl, pitch, c, NV, to_planes);
-        else
-            convert_cell<PB + 1>(q0, pl, pitch, c, NV, to_planes);
+        unsigned long long* q0 = reinterpret_cast<unsigned long long*>(aos) + I.aos_offset[b.parity] + c0 * row;
+        if ((int)threadIdx.x < cnt) {
+            double* q = reinterpret_cast<double*>(to_planes ? q0 : sm) + threadIdx.x * row;
+            if (I.group == 0)
+                convert_cell<PA + 1>(q, pl, pitch, c0 + threadIdx.x, NV, to_planes);
+            else
+                convert_cell<PB + 1>(q, pl, pitch, c0 + threadIdx.x, NV, to_planes);
+        }
+        if (!to_planes) {
+            __syncthreads();
+            for (int k = threadIdx.x; k < cnt * row; k += kThreads) q0[k] = sm[k];
+            __syncthreads();
+        }
     }
 }
 

@@ -53,7 +53,7 @@ struct wcc_batch_ctx {
     long long steps = 0;
     bool initialised = false;
     int sms = 0, max_ctas_per_sm = 1;
-    unsigned grid = 0;  // persistent CTAs of the step kernel
+    unsigned grid = 0;  // CTAs of the step kernel (one per tile, or a grid that walks the tiles)
 
     cudaGraphExec_t gexec = nullptr;
     int g_cur = -1, g_parity = -1, g_chunk = 0;
@@ -155,6 +155,12 @@ cudaError_t launch(wcc_batch_ctx* b, int kind, const BatchArgs& a, double* aos, 
         case WCC_BURGERS: return launch_batch<BURGERS>(b->PA, b->PB, kind, a, aos, to_planes, grid, b->stream);
         default: return launch_batch<EULER>(b->PA, b->PB, kind, a, aos, to_planes, grid, b->stream);
     }
+}
+
+// One CTA per tile of any of the batch's half-step launches.
+unsigned tile_grid(const wcc_batch_ctx* b) {
+    const long long t = std::max(std::max(b->tiles_step[0], b->tiles_step[1]), std::max(b->tiles_pair[0], b->tiles_pair[1]));
+    return (unsigned)std::min<long long>(std::max<long long>(t, 1), 1ll << 30);
 }
 
 unsigned aux_grid(wcc_batch_ctx* b, long long tiles) {
@@ -614,7 +620,7 @@ int wcc_batch_create(wcc_batch* out, int system, int64_t count, const int64_t* N
         default: b->max_ctas_per_sm = batch_blocks_per_sm<EULER>(b->PA, b->PB); break;
     }
     if (b->max_ctas_per_sm < 1) b->max_ctas_per_sm = 1;
-    b->grid = (unsigned)(b->max_ctas_per_sm * b->sms);
+    b->grid = tile_grid(b);
     if (ensure_hist(b, 1024) != WCC_OK || cudaStreamSynchronize(b->stream) != cudaSuccess) {
         std::string m = b->err;
         release(b);
@@ -733,7 +739,7 @@ int wcc_batch_set_grid(wcc_batch b, int ctas) {
     if (!b) return bfail(nullptr, WCC_E_INVAL, "NULL batch");
     DeviceScope ds_(b->device);
     if (ctas < 0) return bfail(b, WCC_E_INVAL, "ctas must be >= 0");
-    b->grid = ctas == 0 ? (unsigned)(b->max_ctas_per_sm * b->sms) : (unsigned)ctas;
+    b->grid = ctas == 0 ? tile_grid(b) : (unsigned)ctas;
     return WCC_OK;
 }
 
@@ -755,9 +761,7 @@ int wcc_batch_autotune(wcc_batch b, double cfl, int* ctas_out) {
     std::vector<Cand> cand;
     for (int tb = 1; tb <= (b->pairs_compiled ? 2 : 1); ++tb) {
         for (int k = 1; k <= b->max_ctas_per_sm; ++k) cand.push_back({(unsigned)(k * b->sms), tb});
-        const long long tiles = tb == 1 ? std::max(b->tiles_step[0], b->tiles_step[1])
-                                        : std::max(b->tiles_pair[0], b->tiles_pair[1]);
-        cand.push_back({(unsigned)std::min<long long>(tiles, 1ll << 30), tb});
+        cand.push_back({tile_grid(b), tb});
     }
     const int G = b->PB == b->PA ? 1 : 2;
     size_t plane_bytes[2] = {0, 0};

@@ -698,8 +698,12 @@ struct PairBook {
     int cfl_mode;
     int parity;
     DevState* backup;   // batches: the state before the pair, or nullptr
-    unsigned* refused;  // batches: set to 1 when this state refuses the pair, or nullptr
+    unsigned* refused;  // batches: set to pair_mark when this state refuses the pair, or nullptr
 };
+
+// What the refusal flag of a batch holds: the half-steps taken before the
+// refusing launch (all instances have taken as many), and never 0.
+__device__ __forceinline__ unsigned pair_mark(long long step) { return (unsigned)step * 2u + 1u; }
 
 // Bookkeeping of a two-half-step launch after the last CTA of a problem
 // finished (one thread): the pair is taken when the realised CFL number of
@@ -723,7 +727,7 @@ __device__ __forceinline__ void finalize_pair(const PairBook& bk, double dt) {
     const double nu2 = dt * (double)fmid / bk.dx;
     if (!(nu2 <= bk.nu_max)) {
         st->err |= ERR_CFL;
-        if (bk.refused) atomicExch(bk.refused, 1u);
+        if (bk.refused) atomicExch(bk.refused, pair_mark(st->step));
         __threadfence();
         return;
     }

@@ -158,3 +158,21 @@ def test_full_batch_workload_sampled():
         q, dts, _ = _alone(probs[i], nsteps)
         np.testing.assert_allclose(hists[i], dts, rtol=1e-5)
         assert fp32_pair_violation(probs[i], qs[i], q, hists[i]) <= 1.0
+
+
+@pytest.mark.parametrize("grid", [0, 3, 100000])
+def test_refused_pairs_with_any_grid(grid):
+    # a pair refused by one instance leaves every instance untouched also when
+    # many of the launch's tiles start after the refusal (one CTA per tile):
+    # the batch then equals the one that takes single half-steps
+    probs = inputs.batch_workload(400, n_min=256, n_max=4096, seed=11, degrees=(2, 3))
+    with wcc.Batch(probs, tb_depth=2, tb_cfl_growth=-1.0) as a, wcc.Batch(probs) as b:
+        for s in (a, b):
+            s.set_initial()
+            s.set_grid(grid)
+            s.step(12, CFL)
+        assert a.tb_stats() == (0, 6)
+        for i in (0, 7, 399):
+            assert np.array_equal(a.dt_history(i), b.dt_history(i))
+        for qa, qb in zip(a.get_dofs(), b.get_dofs()):
+            assert np.array_equal(qa, qb)
