@@ -52,17 +52,13 @@ __device__ __forceinline__ unsigned long long warp_max_key(unsigned long long k)
     return ((unsigned long long)m << 32) | lo;
 }
 
-// dt = cfl dx / amax and lam = dt / dx of the next half-step.  FP64 kernels
-// take the quotients from a reciprocal with the remainder added back: the
-// bookkeeping is a serial chain at the end of a launch, where a warp's FP64
-// instruction takes 64 cycles and a division nine of them.  The FP32 kernels
-// keep the divisions (the other form costs them registers: two half-steps per
-// launch at P = 2 ran 1.3 % slower).
-template <bool F32>
-__device__ __forceinline__ void next_step(DevState* st, double cfl, double dx, double inv_dx, double amax) {
-    double dt, lam;
+// dt = cfl dx / amax and lam = dt / dx, quotients from a reciprocal with the
+// remainder added back: on the serial path between half-steps a warp's FP64
+// instruction takes 64 cycles and a division nine of them.
+__device__ __forceinline__ void cfl_quotients(double cfl, double dx, double inv_dx, double amax, double& dt,
+                                              double& lam) {
     const double x = cfl * dx;
-    if (!F32 && mid_range(amax) && mid_range(x) && mid_range(inv_dx)) {
+    if (mid_range(amax) && mid_range(x) && mid_range(inv_dx)) {
         const d3 a(amax), n(x), ix(inv_dx);
         const d3 r = recip(a), q = n * r;
         const d3 t = fma(fma(-q, a, n), r, q);
@@ -73,9 +69,23 @@ __device__ __forceinline__ void next_step(DevState* st, double cfl, double dx, d
         dt = x / amax;
         lam = dt / dx;
     }
+}
+
+// The size of the next half-step into the state.  (The FP32 kernels of one
+// half-step per launch keep the divisions: the form above costs them
+// registers, and two half-steps per launch at P = 2 ran 1.3 % slower.)
+template <bool F32>
+__device__ __forceinline__ void next_step(DevState* st, double cfl, double dx, double inv_dx, double amax) {
+    double dt, lam;
+    if constexpr (F32) {
+        dt = cfl * dx / amax;
+        lam = dt / dx;
+        split_to_floats(lam, st->next_lam_hi, st->next_lam_lo);
+    } else {
+        cfl_quotients(cfl, dx, inv_dx, amax, dt, lam);
+    }
     st->next_dt = dt;
     st->next_lam = lam;
-    if (F32) split_to_floats(lam, st->next_lam_hi, st->next_lam_lo);
     st->next_cfl = cfl;
 }
 
@@ -165,34 +175,42 @@ __device__ __forceinline__ void finish_halfstep(T speed, unsigned err, double dt
                              args.cfl_mode, args.cfl, args.dx, args.inv_dx);
 }
 
-template <int SYS, int P>
-__global__ void __launch_bounds__(kThreads) halfstep_fp64(const StepArgs args) {
+// Where one FP64 tile reads and writes.
+struct TileIO64 {
+    const double* in64;
+    double* out64;
+    long long pitch;
+    long long n_old;
+    long long n_new;
+    long long first_new;
+    int parity;
+};
+
+// One tile of the FP64 half-step: kThreads parents (stage index io.first_new +
+// t - parity), kTile new cells.  step() gives the half-step's size.  speed
+// receives the thread's new cell's speed (unchanged outside the stage); the
+// caller synchronises the block before rec is written again.
+template <int SYS, int P, class Step>
+__device__ __forceinline__ void fp64_tile(const TileIO64& io, Step&& step, const StepArgs& args,
+                                          double (*rec)[kThreads], double& speed, unsigned& err) {
     constexpr int NV = nvars(SYS);
     constexpr int K = P + 1;
-    constexpr int NREC = NV * (P + 3);
-    __shared__ double rec[NREC][kThreads];
-
     const int t = threadIdx.x;
-    const long long first_new = (long long)blockIdx.x * kTile;
-
-    pdl_begin();
-    const StepSize z = step_size(args);
-    const double dt = z.dt;
-    const double lam = z.lam;
 
     // ---- phase 1: parent record of parent slot t
     {
-        const long long p = parent_index(first_new + t - (args.parity ? 1 : 0), args.n_old, args.bc);
+        const long long p = parent_index(io.first_new + t - (io.parity ? 1 : 0), io.n_old, args.bc);
         d3 c[NV][K];
         sfor<0, NV>([&](auto V) {
             constexpr int v = decltype(V)::value;
             sfor<0, K>([&](auto Ki) {
                 constexpr int k = decltype(Ki)::value;
-                c[v][k] = d3::reg(args.in64[(long long)(v * K + k) * args.pitch + p]);
+                c[v][k] = d3::reg(io.in64[(long long)(v * K + k) * io.pitch + p]);
             });
         });
+        const StepSize& z = step();  // after the parents' loads have been issued
         ParentRecord<SYS, P, d3> r;
-        parent_record<SYS, P, d3>(c, d3(lam), args, r);
+        parent_record<SYS, P, d3>(c, d3(z.lam), args, r);
         sfor<0, NV>([&](auto V) {
             constexpr int v = decltype(V)::value;
             rec[v][t] = r.A[v].v;
@@ -206,10 +224,8 @@ __global__ void __launch_bounds__(kThreads) halfstep_fp64(const StepArgs args) {
     __syncthreads();
 
     // ---- phase 2: new cell t from parent slots t (left) and t + 1 (right)
-    const long long i = first_new + t;
-    double speed = 0.0;
-    unsigned err = 0u;
-    if (t < kTile && i < args.n_new) {
+    const long long i = io.first_new + t;
+    if (t < kTile && i < io.n_new) {
         d3 e[NV][K], ubar[NV], dl[NV], dr[NV];
         sfor<0, NV>([&](auto V) {
             constexpr int v = decltype(V)::value;
@@ -271,7 +287,7 @@ __global__ void __launch_bounds__(kThreads) halfstep_fp64(const StepArgs args) {
             sfor<0, K>([&](auto Ki) {
                 constexpr int k = decltype(Ki)::value;
                 bad |= not_finite(e[v][k]);
-                __stcs(args.out64 + (long long)(v * K + k) * args.pitch + i, e[v][k].v);
+                __stcs(io.out64 + (long long)(v * K + k) * io.pitch + i, e[v][k].v);
             });
         });
         if (bad) err |= ERR_NONFINITE;
@@ -279,7 +295,19 @@ __global__ void __launch_bounds__(kThreads) halfstep_fp64(const StepArgs args) {
         sfor<0, NV>([&](auto V) { u0[decltype(V)::value] = e[decltype(V)::value][0]; });
         speed = wave_speed<SYS, d3>(u0, args, err).v;
     }
-    finish_halfstep<double>(speed, err, dt, args);
+}
+
+template <int SYS, int P>
+__global__ void __launch_bounds__(kThreads) halfstep_fp64(const StepArgs args) {
+    __shared__ double rec[nvars(SYS) * (P + 3)][kThreads];
+    pdl_begin();
+    const TileIO64 io{args.in64, args.out64, args.pitch, args.n_old, args.n_new,
+                      (long long)blockIdx.x * kTile, args.parity};
+    StepSize z;
+    double speed = 0.0;
+    unsigned err = 0u;
+    fp64_tile<SYS, P>(io, [&]() -> const StepSize& { return z = step_size(args); }, args, rec, speed, err);
+    finish_halfstep<double>(speed, err, z.dt, args);
 }
 
 // Largest characteristic speed of a stage (used once after loading data).

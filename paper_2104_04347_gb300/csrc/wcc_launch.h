@@ -22,6 +22,15 @@ cudaError_t launch_halfstep_mixed_hi(int P, int precision, const StepArgs& args,
 template <int SYS>
 cudaError_t launch_halfstep_pair_hi(int P, int precision, const StepArgs& args, cudaStream_t stream);
 
+// nsteps CFL half-steps (at most kSmallSteps) of a mesh of a few tiles in one
+// launch of a cluster of `ctas` CTAs (wcc_small.cuh; FP64 at every P,
+// FP32-mixed at P <= 4), fewer where t_stop (infinite: none) is reached.  fits not null: no launch, *fits receives how many such
+// clusters the device holds (0: none, or no such kernel).
+template <int SYS>
+cudaError_t launch_small(int P, int precision, const StepArgs& args, int nsteps, double t_stop, int ctas,
+                         cudaStream_t stream, int* fits);
+int small_cluster(int precision, long long n);  // CTAs for stages of at most n cells, 0: too many
+
 // Two half-steps in one launch (FP32 variants, P <= 4; halfstep_mixed2_tb2):
 // args.in32 -> args.out32 with args.n_mid cells in between;
 // grid = ceil(n_new / kTileTB) CTAs.
