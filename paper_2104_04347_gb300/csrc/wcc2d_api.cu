@@ -129,8 +129,6 @@ cudaError_t plan_launches(wcc2d_ctx* h) {
     return cudaSuccess;
 }
 
-int conv_grid(long long n) { return (int)std::min<long long>((n + 255) / 256, 152LL * 16); }
-
 }  // namespace
 
 extern "C" {
@@ -197,7 +195,7 @@ int wcc2d_create(wcc2d_handle* out, int system, int64_t nx, int64_t ny, int P, c
     h->dx = (domain[1] - domain[0]) / (double)nx;
     h->dy = (domain[3] - domain[2]) / (double)ny;
     h->opt = o;
-    h->law = Law2D{o.ax, o.ay, o.gamma, o.alpha, o.eps, o.limiter ? 1 : 0};
+    h->law = make_law2d(o.ax, o.ay, o.gamma, o.alpha, o.eps, o.limiter ? 1 : 0);
     if (o.cuda_stream) {
         h->stream = static_cast<cudaStream_t>(o.cuda_stream);
     } else {
@@ -275,17 +273,8 @@ int wcc2d_set_initial(wcc2d_handle h, const double* dofs, int64_t count) {
     if (count != cx * cy * nd) return fail2(h, WCC_E_INVAL, "count does not match an integer stage");
     WCC2D_CHECK(h, cudaMemcpyAsync(h->staging, dofs, (size_t)count * sizeof(double), cudaMemcpyHostToDevice,
                                    h->stream));
-    const int g = conv_grid(cx * cy * nd);
-    if (h->mixed)
-        WCC2D_CHECK(h, launch_convert2d_mx(h->P, true, h->staging, static_cast<float*>(h->planes[0]), (int)cx, (int)cy,
-                                           h->nv, h->pitch, h->plane, h->stream));
-    else if (h->fp32)
-        aos_to_planes2d<float><<<g, 256, 0, h->stream>>>(h->staging, static_cast<float*>(h->planes[0]), (int)cx,
-                                                         (int)cy, nd, h->pitch, h->plane);
-    else
-        aos_to_planes2d<double><<<g, 256, 0, h->stream>>>(h->staging, static_cast<double*>(h->planes[0]), (int)cx,
-                                                          (int)cy, nd, h->pitch, h->plane);
-    WCC2D_CHECK(h, cudaGetLastError());
+    WCC2D_CHECK(h, launch_convert2d(h->P, h->mixed ? 2 : h->fp32, true, h->staging, h->planes[0], (int)cx, (int)cy, h->nv,
+                                    h->pitch, h->plane, h->stream));
     WCC2D_CHECK(h, cudaMemsetAsync(h->st, 0, sizeof(DevState2D), h->stream));
     if (h->mixed)
         WCC2D_CHECK(h, launch_stage_rate2d_mx(h->system, h->P, static_cast<const float*>(h->planes[0]), h->pitch,
@@ -453,17 +442,8 @@ int wcc2d_get_dofs(wcc2d_handle h, double* dofs, int64_t count) {
     DevState2D s;
     int rc = read_state(h, &s);
     if (rc != WCC_OK) return rc;
-    const int g = conv_grid(cx * cy * nd);
-    if (h->mixed)
-        WCC2D_CHECK(h, launch_convert2d_mx(h->P, false, h->staging, static_cast<float*>(h->planes[h->cur]), (int)cx,
-                                           (int)cy, h->nv, h->pitch, h->plane, h->stream));
-    else if (h->fp32)
-        planes_to_aos2d<float><<<g, 256, 0, h->stream>>>(static_cast<const float*>(h->planes[h->cur]), h->staging,
-                                                         (int)cx, (int)cy, nd, h->pitch, h->plane);
-    else
-        planes_to_aos2d<double><<<g, 256, 0, h->stream>>>(static_cast<const double*>(h->planes[h->cur]), h->staging,
-                                                          (int)cx, (int)cy, nd, h->pitch, h->plane);
-    WCC2D_CHECK(h, cudaGetLastError());
+    WCC2D_CHECK(h, launch_convert2d(h->P, h->mixed ? 2 : h->fp32, false, h->staging, h->planes[h->cur], (int)cx, (int)cy,
+                                    h->nv, h->pitch, h->plane, h->stream));
     h->launches += 1;
     WCC2D_CHECK(h, cudaMemcpyAsync(dofs, h->staging, (size_t)count * sizeof(double), cudaMemcpyDeviceToHost,
                                    h->stream));

@@ -2,8 +2,8 @@
 // CFL rate of a loaded stage, and the conversions between the host layout
 // [row][col][var][q] (FP64) and the device planes.
 //
-// Device layout: plane (v, q) holds u_{kx,ly} of variable v (q = position of
-// (k, l)) for every cell, row-major with `pitch` elements per row; planes are
+// Device layout: plane (v, q) holds the Taylor coefficient e_kl = u_{kx,ly} /
+// (k! l!) of variable v (q = position of (k, l)) for every cell, row-major with `pitch` elements per row; planes are
 // `plane` elements apart.  T is double (FP64 path) or float (FP32 path).
 //
 // The half-step kernel runs one CTA of TW threads per strip of TW - 1 new
@@ -19,6 +19,8 @@
 #include <algorithm>
 
 #include "wcc2d_scheme.cuh"
+#include "wcc_convert.cuh"
+#include "wcc_halfstep.cuh"
 #include "wcc_pdl.cuh"
 
 namespace wcc2d {
@@ -65,16 +67,26 @@ __device__ __forceinline__ int parent_index(int j, int n_old, int bc) {
 
 // Reads parent records from the ring: vertex r = 0..3 is parent column t
 // (r = 0, 3) or t + 1 (r = 1, 2) of the lower (r = 0, 1) or upper row.
+// Compute type of a stage type, and values between the two.
+template <class T>
+using compute_t = std::conditional_t<sizeof(T) == 8, d3, float>;
+__device__ __forceinline__ float from_memory(float x) { return x; }
+__device__ __forceinline__ d3 from_memory(double x) { return d3::reg(x); }
+__device__ __forceinline__ float to_memory(float x) { return x; }
+__device__ __forceinline__ double to_memory(d3 x) { return x.v; }
+
 template <class T, int TW, int NV, int NQ1>
 struct RingReader {
+    using R = compute_t<T>;
     const T* lo;
     const T* hi;
     int t;
-    __device__ __forceinline__ T get(int r, int f) const {
-        return r == 0 ? lo[f * TW + t] : r == 1 ? lo[f * TW + t + 1] : r == 2 ? hi[f * TW + t + 1] : hi[f * TW + t];
+    __device__ __forceinline__ R get(int r, int f) const {
+        return from_memory(r == 0 ? lo[f * TW + t] : r == 1 ? lo[f * TW + t + 1] : r == 2 ? hi[f * TW + t + 1]
+                                                                                       : hi[f * TW + t]);
     }
-    __device__ __forceinline__ T c(int r, int v) const { return get(r, v * 4 + r); }
-    __device__ __forceinline__ T V(int r, int v, int q) const { return get(r, NV * 4 + v * NQ1 + q); }
+    __device__ __forceinline__ R c(int r, int v) const { return get(r, v * 4 + r); }
+    __device__ __forceinline__ R V(int r, int v, int q) const { return get(r, NV * 4 + v * NQ1 + q); }
 };
 
 template <int SYS, int P>
@@ -100,33 +112,36 @@ __device__ __forceinline__ double step_dt2d(const Step2D& a) {
     return s_dt;
 }
 
-// Block-wide max of the rate and OR of the error bits, one atomic each per
-// CTA; the CTA that finishes last does the half-step's bookkeeping.
+// Block-wide max of the rate (on the bits of the non-negative numbers) and OR
+// of the error bits, one atomic each per CTA; the CTA that finishes last does
+// the half-step's bookkeeping.
 template <class T, int NT>
 __device__ __forceinline__ void finish2d(T rate, unsigned err, double dt, const Step2D& a) {
-    __shared__ double s_max[NT / 32];
+    using Key = decltype(wcc::speed_key(rate));
+    __shared__ Key s_max[NT / 32];
     __shared__ unsigned s_err[NT / 32];
-    double r = (double)rate;
-    if (r != r) {
-        r = INFINITY;
+    if (rate != rate) {
+        rate = (T)INFINITY;
         err |= ERR_NONFINITE;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) r = fmax(r, __shfl_xor_sync(0xffffffffu, r, o));
+    const Key key = wcc::warp_max_key(wcc::speed_key(rate));
     err = __reduce_or_sync(0xffffffffu, err);
     if ((threadIdx.x & 31) == 0) {
-        s_max[threadIdx.x >> 5] = r;
+        s_max[threadIdx.x >> 5] = key;
         s_err[threadIdx.x >> 5] = err;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        double m = s_max[0];
+        Key mk = s_max[0];
         unsigned e = s_err[0];
 #pragma unroll
         for (int w = 1; w < NT / 32; ++w) {
-            m = fmax(m, s_max[w]);
+            mk = s_max[w] > mk ? s_max[w] : mk;
             e |= s_err[w];
         }
+        double m;
+        if constexpr (sizeof(T) == 8) m = __longlong_as_double((long long)mk);
+        else m = (double)__uint_as_float(mk);
         DevState2D* st = a.st;
         atomicMax(&st->rate_bits[a.parity ^ 1], (unsigned long long)__double_as_longlong(m));
         if (e) atomicOr(&st->err, e);
@@ -156,6 +171,11 @@ constexpr int min_ctas2d() {
     return sizeof(T) == 4 ? 4 : 1;
 }
 
+// The FP64 kernel is bound by the FP64 pipe: Euler P = 3 issues about 2100 FP64
+// instructions per cell, all three-register DFMAs (about 3000 of every form in
+// the derivative form with IEEE divisions): 192 x 192 0.42 -> 0.25 ms per
+// half-step.  The FP32 kernels are bound by issue and dependency latency at 12 to
+// 16 warps per SM.
 template <int SYS, int P, class T, int TW>
 __global__ void __launch_bounds__(TW, min_ctas2d<T>()) halfstep2d(const Step2D a) {
     constexpr int NV = nvars(SYS), NQ = nq(P), NQ1 = nq(P - 1);
@@ -171,8 +191,9 @@ __global__ void __launch_bounds__(TW, min_ctas2d<T>()) halfstep2d(const Step2D a
 
     wcc::pdl_begin();
     const double dt = step_dt2d(a);
-    const T lamx = (T)(dt * a.inv_dx), lamy = (T)(dt * a.inv_dy);
-    const T idx = (T)a.inv_dx, idy = (T)a.inv_dy;
+    using R = compute_t<T>;
+    const R lamx = (R)(dt * a.inv_dx), lamy = (R)(dt * a.inv_dy);
+    const R idx = (R)a.inv_dx, idy = (R)a.inv_dy;
 
     const T* in = static_cast<const T*>(a.in);
     T* out = static_cast<T*>(a.out);
@@ -191,42 +212,51 @@ __global__ void __launch_bounds__(TW, min_ctas2d<T>()) halfstep2d(const Step2D a
                 cell = 0;
             }
 #endif
-            T q[NV][NQ];
+            R q[NV][NQ];
 #pragma unroll
             for (int v = 0; v < NV; ++v)
 #pragma unroll
-                for (int qq = 0; qq < NQ; ++qq) q[v][qq] = in[(long long)(v * NQ + qq) * a.plane + cell];
-            Parent<SYS, P, T> par;
-            parent_terms<SYS, P, T>(q, lamx, lamy, a.law, par);
+                for (int qq = 0; qq < NQ; ++qq) q[v][qq] = from_memory(in[(long long)(v * NQ + qq) * a.plane + cell]);
+            Parent<SYS, P, R> par;
+            parent_terms<SYS, P, R>(q, lamx, lamy, a.law, par);
             T* r = ring + (s & 1) * NF * TW;
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
 #pragma unroll
-                for (int k = 0; k < 4; ++k) r[(v * 4 + k) * TW + t] = par.c[v][k];
+                for (int k = 0; k < 4; ++k) r[(v * 4 + k) * TW + t] = to_memory(par.c[v][k]);
 #pragma unroll
-                for (int qq = 0; qq < NQ1; ++qq) r[(NV * 4 + v * NQ1 + qq) * TW + t] = par.V[v][qq];
+                for (int qq = 0; qq < NQ1; ++qq) r[(NV * 4 + v * NQ1 + qq) * TW + t] = to_memory(par.V[v][qq]);
             }
         }
         __syncthreads();
         if (s >= 1 && t < TW - 1 && i0 + t < a.nx_new) {
             const RingReader<T, TW, NV, NQ1> rd{ring + ((s - 1) & 1) * NF * TW, ring + (s & 1) * NF * TW, t};
-            T D[NV][NQ], ub[NV];
-            linear_cell<SYS, P, T>(rd, D, ub);
+            // FP64 Euler: the first derivatives after the projection (limit_euler)
+            constexpr bool kLate = SYS == EULER && sizeof(T) == 8;
+            R D[NV][NQ], ub[NV], vv[NV][4];
+            linear_cell<SYS, P, kLate ? 2 : 1, R>(rd, D, ub);
+#pragma unroll
+            for (int v = 0; v < NV; ++v)
+#pragma unroll
+                for (int r = 0; r < 4; ++r) vv[v][r] = rd.V(r, v, 0) - ub[v];
+            bool limited = false;
             if (a.law.limiter) {
                 if constexpr (SYS == EULER) {
-                    T vv[4][4];
-#pragma unroll
-                    for (int v = 0; v < 4; ++v)
-#pragma unroll
-                        for (int r = 0; r < 4; ++r) vv[v][r] = rd.V(r, v, 0);
-                    if (!limit_euler<P, T>(D, ub, vv, lamx, lamy, a.law)) err |= ERR_POSITIVITY;
+                    limited = limit_euler<P, R>(D, ub, vv, lamx, lamy, a.law);
+                    if (!limited) err |= ERR_POSITIVITY;
                 } else {
-                    T vv[4];
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) vv[r] = rd.V(r, 0, 0);
-                    limit_scalar<P, T>(D[0], ub[0], vv, a.law);
+                    limit_scalar<P, R>(D[0], vv[0], a.law, ub[0]);
                 }
             }
+            if constexpr (kLate) {
+                if (!limited) {
+#pragma unroll
+                    for (int v = 0; v < NV; ++v) first_derivatives<P, R>(D[v], vv[v]);
+                }
+            }
+            // the limiter keeps the cell average (every candidate has mean ubar)
+#pragma unroll
+            for (int v = 0; v < NV; ++v) D[v][0] = ub[v] - even_correction<P, R>(D[v]);
             const long long cell = (long long)(j0 + s - 1) * a.pitch + (i0 + t);
             bool store = true;
 #ifdef WCC2D_BOUNDS_CHECK
@@ -239,17 +269,18 @@ __global__ void __launch_bounds__(TW, min_ctas2d<T>()) halfstep2d(const Step2D a
 #pragma unroll
                 for (int v = 0; v < NV; ++v)
 #pragma unroll
-                    for (int qq = 0; qq < NQ; ++qq) out[(long long)(v * NQ + qq) * a.plane + cell] = D[v][qq];
+                    for (int qq = 0; qq < NQ; ++qq) out[(long long)(v * NQ + qq) * a.plane + cell] = to_memory(D[v][qq]);
             }
-            T centre[NV];
+            R centre[NV];
 #pragma unroll
             for (int v = 0; v < NV; ++v) centre[v] = D[v][0];
-            const T rate = cfl_rate<SYS, T>(centre, a.law, idx, idy);
-            if (rate != rate) {
-                err |= (SYS == EULER && ub[0] == ub[0]) ? ERR_POSITIVITY : ERR_NONFINITE;
+            const R rate = cfl_rate<SYS, R>(centre, a.law, idx, idy);
+            if (is_nan(rate)) {
+                err |= (SYS == EULER && !is_nan(ub[0])) ? ERR_POSITIVITY : ERR_NONFINITE;
                 rate_max = (T)INFINITY;
             } else {
-                rate_max = rate > rate_max ? rate : rate_max;
+                const T r = to_memory(rate);
+                rate_max = wcc::speed_key(r) > wcc::speed_key(rate_max) ? r : rate_max;
             }
         }
         __syncthreads();
@@ -257,59 +288,163 @@ __global__ void __launch_bounds__(TW, min_ctas2d<T>()) halfstep2d(const Step2D a
     finish2d<T, TW>(rate_max, err, dt, a);
 }
 
+// A warp's largest CFL rate of a loaded stage into rate_bits[0] (and the error bits).
+__device__ __forceinline__ void post_rate(double r, unsigned err, DevState2D* st) {
+    const unsigned long long key = wcc::warp_max_key(wcc::speed_key(r));
+    err = __reduce_or_sync(0xffffffffu, err);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(&st->rate_bits[0], key);
+        if (err) atomicOr(&st->err, err);
+    }
+}
+
 // CFL rate of a loaded stage into rate_bits[0] (and the error bits).
 template <int SYS, class T>
 __global__ void __launch_bounds__(256) stage_rate2d(const T* planes, long long pitch, long long plane, int nx, int ny,
                                                     int nq_, Law2D law, double dx, double dy, DevState2D* st) {
     constexpr int NV = nvars(SYS);
+    using R = compute_t<T>;
     T m = 0;
     unsigned err = 0;
     const long long n = (long long)nx * ny;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
         const long long cell = (c / nx) * pitch + (c % nx);
-        T centre[NV];
+        R centre[NV];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) centre[v] = planes[(long long)(v * nq_) * plane + cell];
-        const T r = cfl_rate<SYS, T>(centre, law, (T)(1.0 / dx), (T)(1.0 / dy));
-        if (r != r) {
+        for (int v = 0; v < NV; ++v) centre[v] = from_memory(planes[(long long)(v * nq_) * plane + cell]);
+        const R r = cfl_rate<SYS, R>(centre, law, (R)(1.0 / dx), (R)(1.0 / dy));
+        if (is_nan(r)) {
             err |= SYS == EULER ? ERR_POSITIVITY : ERR_NONFINITE;
             m = (T)INFINITY;
-        } else if (r > m) {
-            m = r;
+        } else if (to_memory(r) > m) {
+            m = to_memory(r);
         }
     }
-    double r = (double)m;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) r = fmax(r, __shfl_xor_sync(0xffffffffu, r, o));
-    err = __reduce_or_sync(0xffffffffu, err);
-    if ((threadIdx.x & 31) == 0) {
-        atomicMax(&st->rate_bits[0], (unsigned long long)__double_as_longlong(r));
-        if (err) atomicOr(&st->err, err);
+    post_rate((double)m, err, st);
+}
+
+// Conversions between the host layout [row][col][v][q] (FP64 scaled derivatives,
+// in a staging buffer) and the planes.  A CTA takes kConvCells cells of a row:
+// its host-layout side is one run of doubles, its plane side a run per plane,
+// and the transposition goes through shared memory, so that both sides move
+// whole sectors.  (One thread per cell, stepping through its cell's doubles:
+// 158 us to the planes and 527 us back at 1024 x 1024, FP32-mixed, P = 3; about
+// 110 and 190 us this way.)
+// FP32 stages are converted on the FP32 and integer pipes (wcc_convert.cuh).
+constexpr int kConvCells = 64, kConvThreads = 256;
+
+// 1/(k! l!) and k! l! of position q
+__host__ __device__ constexpr double fact_q(int q) { return factd(qk_of(q)) * factd(ql_of(q)); }
+
+// One variable of one cell, d its scaled derivatives (bit patterns), put(plane, x):
+// FP64 (T = double), FP32 point values, or FP32-mixed (cell average as a
+// float-float pair in planes 0 and -1).
+template <int P, bool MX, class T, class Put>
+__device__ __forceinline__ void variable_to_planes(const unsigned long long* d, Put&& put) {
+    if constexpr (sizeof(T) == 8) {
+        unroll<nq(P)>([&](auto qc) {
+            constexpr double w = 1.0 / fact_q(qc);
+            const double x = __longlong_as_double((long long)d[qc]);
+            put(qc, w == 1.0 ? x : x * w);
+        });
+    } else {
+        ff e[nq(P)];
+        unroll<nq(P)>([&](auto qc) {
+            constexpr wcc::ffc w = wcc::ffc_of(1.0 / fact_q(qc));
+            e[qc] = wcc::split_double_bits(d[qc]);
+            if constexpr (fact_q(qc) != 1.0) e[qc] = wcc::ff_mul_c(e[qc], w);
+            else e[qc] = wcc::fast_two_sum(e[qc].hi, e[qc].lo);
+        });
+        if constexpr (MX) {
+            ff u = e[0];
+            if constexpr (P >= 2) {
+                constexpr wcc::ffc w = wcc::ffc_of(1.0 / 12.0);
+                u = wcc::ff_add(u, wcc::ff_mul_c(wcc::ff_add(e[qidx(2, 0)], e[qidx(0, 2)]), w));
+            }
+            u = wcc::fast_two_sum(u.hi, u.lo);
+            put(0, u.hi);
+            put(-1, u.lo);
+        } else {
+            put(0, e[0].hi);
+        }
+        unroll<nq(P) - 1>([&](auto qc) { put(qc + 1, e[qc + 1].hi); });
     }
 }
 
-// host [row][col][v][q] FP64 (staging) -> planes of T, and back; one thread
-// per (cell, value), consecutive threads on consecutive cells of a plane
-template <class T>
-__global__ void aos_to_planes2d(const double* aos, T* planes, int nx, int ny, int nd, long long pitch,
-                                long long plane) {
-    const long long n = (long long)nx * ny;
-    for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < n * nd;
-         g += (long long)gridDim.x * blockDim.x) {
-        const long long f = g / n, c = g % n;
-        planes[f * plane + (c / nx) * pitch + (c % nx)] = (T)aos[c * nd + f];
+// The way back: get(plane) reads, d receives the scaled derivatives.
+template <int P, bool MX, class T, class Get>
+__device__ __forceinline__ void planes_to_variable(Get&& get, unsigned long long* d) {
+    if constexpr (sizeof(T) == 8) {
+        unroll<nq(P)>([&](auto qc) {
+            const double x = get(qc);
+            d[qc] = (unsigned long long)__double_as_longlong(fact_q(qc) == 1.0 ? x : x * fact_q(qc));
+        });
+    } else {
+        float e[nq(P)];
+        unroll<nq(P) - 1>([&](auto qc) {
+            constexpr int i = qc + 1;
+            e[i] = get(i);
+            d[i] = wcc::float_times_exact<(unsigned)fact_q(i)>(e[i]);
+        });
+        if constexpr (MX) {
+            ff u{get(0), get(-1)};
+            if constexpr (P >= 2) {
+                constexpr wcc::ffc w = wcc::ffc_of(1.0 / 12.0);
+                u = wcc::ff_sub(u, wcc::ff_mul_c(wcc::two_sum(e[qidx(2, 0)], e[qidx(0, 2)]), w));
+            }
+            d[0] = (unsigned long long)__double_as_longlong(
+                __longlong_as_double((long long)wcc::float_times_exact<1>(u.hi)) +
+                __longlong_as_double((long long)wcc::float_times_exact<1>(u.lo)));
+        } else {
+            d[0] = wcc::float_times_exact<1>(get(0));
+        }
     }
 }
 
-template <class T>
-__global__ void planes_to_aos2d(const T* planes, double* aos, int nx, int ny, int nd, long long pitch,
-                                long long plane) {
-    const long long n = (long long)nx * ny;
-    for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < n * nd;
-         g += (long long)gridDim.x * blockDim.x) {
-        const long long f = g / n, c = g % n;
-        aos[c * nd + f] = (double)planes[f * plane + (c / nx) * pitch + (c % nx)];
+template <int P, bool MX, class T, bool TO_PLANES>
+__global__ void __launch_bounds__(kConvThreads) convert2d(double* aos, T* planes, int nx, int ny, int nv,
+                                                          long long pitch, long long plane) {
+    constexpr int NQ = nq(P), MAXROW = 4 * NQ;
+    __shared__ unsigned long long sm[kConvCells * (MAXROW | 1)];  // odd row length: no bank conflicts
+    const int nd = nv * NQ, row = nd | 1;
+    const int tiles_x = (nx + kConvCells - 1) / kConvCells;
+    const long long tiles = (long long)tiles_x * ny;
+    unsigned long long* host = reinterpret_cast<unsigned long long*>(aos);
+    for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int j = (int)(tile / tiles_x), i0 = (int)(tile % tiles_x) * kConvCells;
+        const int cnt = min(kConvCells, nx - i0);
+        unsigned long long* run = host + ((long long)j * nx + i0) * nd;
+        if constexpr (TO_PLANES) {
+            for (int i = threadIdx.x; i < cnt * nd; i += kConvThreads) sm[(i / nd) * row + i % nd] = run[i];
+            __syncthreads();
+        }
+        for (int i = threadIdx.x; i < kConvCells * nv; i += kConvThreads) {
+            const int c = i % kConvCells, v = i / kConvCells;
+            if (c >= cnt) continue;
+            T* p = planes + (long long)j * pitch + i0 + c;
+            auto at = [&](int qq) -> T& { return p[(long long)(qq < 0 ? nv * NQ + v : v * NQ + qq) * plane]; };
+            unsigned long long* d = sm + c * row + v * NQ;
+            if constexpr (TO_PLANES) variable_to_planes<P, MX, T>(d, [&](int qq, T x) { at(qq) = x; });
+            else planes_to_variable<P, MX, T>([&](int qq) { return at(qq); }, d);
+        }
+        __syncthreads();
+        if constexpr (!TO_PLANES) {
+            for (int i = threadIdx.x; i < cnt * nd; i += kConvThreads) run[i] = sm[(i / nd) * row + i % nd];
+            __syncthreads();
+        }
     }
+}
+
+template <int P, bool MX, class T>
+cudaError_t launch_convert2d_t(bool to_planes, double* aos, void* planes, int nx, int ny, int nv, long long pitch,
+                               long long plane, cudaStream_t stream) {
+    const long long tiles = (long long)((nx + kConvCells - 1) / kConvCells) * ny;
+    const int grid = (int)std::min<long long>(tiles, 152LL * 8);
+    if (to_planes)
+        convert2d<P, MX, T, true><<<grid, kConvThreads, 0, stream>>>(aos, static_cast<T*>(planes), nx, ny, nv, pitch, plane);
+    else
+        convert2d<P, MX, T, false><<<grid, kConvThreads, 0, stream>>>(aos, static_cast<T*>(planes), nx, ny, nv, pitch, plane);
+    return cudaGetLastError();
 }
 
 // CTA width of the half-step: 64 threads for FP64, 128 for FP32, narrowed
@@ -340,7 +475,7 @@ struct StripPlan {
 // 64 cycles whatever else runs, so the slots are the 4 schedulers per SM and
 // the unit is the warp; strips of one warp are taken where they shorten the
 // longest chain (192 x 192 Euler, P = 3: 48 CTAs of 64 threads and 16 rows
-// 1.87 ms, 455 of 32 threads and 3 rows 0.42 ms).
+// 1.87 ms, 455 of 32 threads and 3 rows 0.42 ms with the same arithmetic).
 inline StripPlan plan_strips(int tw, bool fp64, int resident, int sms, int nx_new, int ny_new) {
     StripPlan best{16, 0};
     double best_cost = 1e300;
@@ -462,6 +597,10 @@ struct RingReaderMx {
     }
 };
 
+// Bound by instruction issue (12 warps per SM: 168 registers and the 46 KB ring);
+// Cauchy products without binomial weights, edge fluxes by parity, two
+// residuals instead of four and float constants took Euler P = 3 at 1024 x 1024
+// from 0.200 to 0.167 ms per half-step.
 template <int SYS, int P, int TW>
 __global__ void __launch_bounds__(TW, 4) halfstep2d_mx(const Step2D a) {
     constexpr int NV = nvars(SYS), NQ = nq(P), NQ1 = nq(P - 1);
@@ -504,7 +643,7 @@ __global__ void __launch_bounds__(TW, 4) halfstep2d_mx(const Step2D a) {
                 q[v][0] = 0.f;
 #pragma unroll
                 for (int qq = 1; qq < NQ; ++qq) q[v][qq] = in[(long long)(v * NQ + qq) * a.plane + cell];
-                u00[v] = wcc::ff_add(ub[v], -even_correction<P>(q[v]));
+                u00[v] = wcc::ff_add(ub[v], -even_correction<P, float>(q[v]));
                 q[v][0] = u00[v].hi;
             }
             Parent<SYS, P, float, true> par;
@@ -514,26 +653,19 @@ __global__ void __launch_bounds__(TW, 4) halfstep2d_mx(const Step2D a) {
             float* r = ring + (s & 1) * NF * TW;
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
-                // quarter averages: ubar/4 +- ox +- oy +- oxy with the signs of
-                // RU, LU, LD, RD (vertex roles 1..4), plus the edge fluxes
-                // hx f_U = tx, hx f_D = bx, hy g_R = ry, hy g_L = ly:
-                //   c0 = q4 + ox + oy + oxy + tx + ry,  c1 = q4 - ox + oy - oxy - tx + ly,
-                //   c2 = q4 - ox - oy + oxy - bx - ly,  c3 = q4 + ox - oy - oxy + bx - ry.
-                // The O(1) parts (q4 and the leading flux terms hx f(u_00),
-                // hy g(u_00)) are added exactly, the float parts (the odd
-                // terms and the flux corrections) join the low parts.  c3 is
-                // taken as ubar - c0 - c1 - c2, so the parent's shares add up
-                // to its ubar to float-float rounding.
-                const float ox = 0.25f * par.odd[v][0], oy = 0.25f * par.odd[v][1], oxy = 0.25f * par.odd[v][2];
-                const float sxy = ox + oy, dxy = ox - oy;
+                // the shares a +- p +- q +- r with a = ubar/4 and the leading
+                // flux terms hx f(u_00) in p, hy g(u_00) in q:
+                // the O(1) parts are added exactly, the float parts p, q, r
+                // in one sum, the low parts in another.  c3 is taken as
+                // ubar - c0 - c1 - c2, so the parent's shares add up to its
+                // ubar to float-float rounding.
                 const float q4h = 0.25f * ub[v].hi, q4l = 0.25f * ub[v].lo;
                 const ff hF = ffm_lazy(F[v], hx), hG = ffm_lazy(G[v], hy);
-                const float tl = fmaf(hx, par.fl[v][0], hF.lo), bl = fmaf(hx, par.fl[v][1], hF.lo);
-                const float rl = fmaf(hy, par.fl[v][2], hG.lo), ll = fmaf(hy, par.fl[v][3], hG.lo);
+                const float pr = par.p[v] + par.r[v], mr = par.p[v] - par.r[v];
                 ff c[4];
-                c[0] = ff_sum4(q4h, hF.hi, hG.hi, sxy + oxy, q4l + (tl + rl));
-                c[1] = ff_sum4(q4h, -hF.hi, hG.hi, -(dxy + oxy), q4l + (ll - tl));
-                c[2] = ff_sum4(q4h, -hF.hi, -hG.hi, oxy - sxy, q4l - (bl + ll));
+                c[0] = ff_sum4(q4h, hF.hi, hG.hi, par.q[v] + pr, q4l + (hF.lo + hG.lo));
+                c[1] = ff_sum4(q4h, -hF.hi, hG.hi, par.q[v] - pr, q4l + (hG.lo - hF.lo));
+                c[2] = ff_sum4(q4h, -hF.hi, -hG.hi, -(par.q[v] + mr), q4l - (hF.lo + hG.lo));
                 c[3] = ff_rest3(ub[v], c[0], c[1], c[2]);
                 float2* r2 = reinterpret_cast<float2*>(r);
 #pragma unroll
@@ -551,30 +683,20 @@ __global__ void __launch_bounds__(TW, 4) halfstep2d_mx(const Step2D a) {
             ff ub[NV];
             linear_cell_mx<SYS, P>(rd, D, ub);
             if (a.law.limiter) {
-                // deviation form: the point value and the vertex values less
-                // the average, taken in float-float and rounded, so that the
+                // deviation form: the vertex values less the average, taken
+                // from the float-float pairs and rounded, so that the
                 // limiter's slopes and residuals near smooth extrema are not
-                // float cancellations of O(1) values; the limited point value
-                // comes back as a deviation
+                // float cancellations of O(1) values
+                float vv[NV][4];
+#pragma unroll
+                for (int v = 0; v < NV; ++v)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) vv[v][k] = ff_close_diff(rd.v00(k, v), ub[v]);
                 if constexpr (SYS == EULER) {
-                    float vv[4][4], ubf[4];
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) {
-                        ubf[v] = ub[v].hi;
-                        D[v][0] = -even_correction<P>(D[v]);
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) vv[v][k] = wcc::ff_sub(rd.v00(k, v), ub[v]).hi;
-                    }
-                    if (!limit_euler<P, float, true>(D, ubf, vv, lamx, lamy, a.law)) err |= ERR_POSITIVITY;
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) D[v][0] += ubf[v];
+                    const float ubf[4] = {ub[0].hi, ub[1].hi, ub[2].hi, ub[3].hi};
+                    if (!limit_euler<P, float>(D, ubf, vv, lamx, lamy, a.law)) err |= ERR_POSITIVITY;
                 } else {
-                    float vv[4];
-                    D[0][0] = -even_correction<P>(D[0]);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) vv[k] = wcc::ff_sub(rd.v00(k, 0), ub[0]).hi;
-                    limit_scalar<P, float>(D[0], 0.f, vv, a.law);
-                    D[0][0] += ub[0].hi;
+                    limit_scalar<P, float>(D[0], vv[0], a.law, 0.f);
                 }
             }
             // the limiter keeps the cell average (every candidate has mean ubar)
@@ -588,7 +710,7 @@ __global__ void __launch_bounds__(TW, 4) halfstep2d_mx(const Step2D a) {
             }
             float centre[NV];
 #pragma unroll
-            for (int v = 0; v < NV; ++v) centre[v] = D[v][0];
+            for (int v = 0; v < NV; ++v) centre[v] = wcc::ff_add(ub[v], -even_correction<P, float>(D[v])).hi;
             const float rate = cfl_rate<SYS, float>(centre, a.law, idx, idy);
             if (rate != rate) {
                 err |= (SYS == EULER && ub[0].hi == ub[0].hi) ? ERR_POSITIVITY : ERR_NONFINITE;
@@ -600,56 +722,6 @@ __global__ void __launch_bounds__(TW, 4) halfstep2d_mx(const Step2D a) {
         __syncthreads();
     }
     finish2d<float, TW>(rate_max, err, dt, a);
-}
-
-// host [row][col][v][q] FP64 point values and derivatives <-> FP32-mixed
-// planes; one thread per cell (set-up and read-back only)
-template <int P>
-__global__ void aos_to_planes2d_mx(const double* aos, float* planes, int nx, int ny, int nv, long long pitch,
-                                   long long plane) {
-    constexpr int NQ = nq(P);
-    const long long n = (long long)nx * ny;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
-        const long long cell = (c / nx) * pitch + (c % nx);
-        for (int v = 0; v < nv; ++v) {
-            const double* d = aos + (c * nv + v) * NQ;
-            double ub = d[0];
-            unroll<P + 1>([&](auto kc) {
-                unroll<P + 1 - kc>([&](auto lc) {
-                    constexpr int k = kc, l = lc;
-                    if constexpr (k + l > 0 && !(k & 1) && !(l & 1))
-                        ub += pow2m(k) / factd(k + 1) * pow2m(l) / factd(l + 1) * d[qidx(k, l)];
-                });
-            });
-            const float hi = (float)ub;
-            planes[(long long)(v * NQ) * plane + cell] = hi;
-            planes[(long long)(nv * NQ + v) * plane + cell] = (float)(ub - (double)hi);
-            for (int qq = 1; qq < NQ; ++qq) planes[(long long)(v * NQ + qq) * plane + cell] = (float)d[qq];
-        }
-    }
-}
-
-template <int P>
-__global__ void planes_to_aos2d_mx(const float* planes, double* aos, int nx, int ny, int nv, long long pitch,
-                                   long long plane) {
-    constexpr int NQ = nq(P);
-    const long long n = (long long)nx * ny;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
-        const long long cell = (c / nx) * pitch + (c % nx);
-        for (int v = 0; v < nv; ++v) {
-            double* d = aos + (c * nv + v) * NQ;
-            for (int qq = 1; qq < NQ; ++qq) d[qq] = (double)planes[(long long)(v * NQ + qq) * plane + cell];
-            double u = (double)planes[(long long)(v * NQ) * plane + cell] + (double)planes[(long long)(nv * NQ + v) * plane + cell];
-            unroll<P + 1>([&](auto kc) {
-                unroll<P + 1 - kc>([&](auto lc) {
-                    constexpr int k = kc, l = lc;
-                    if constexpr (k + l > 0 && !(k & 1) && !(l & 1))
-                        u -= pow2m(k) / factd(k + 1) * pow2m(l) / factd(l + 1) * d[qidx(k, l)];
-                });
-            });
-            d[0] = u;
-        }
-    }
 }
 
 // CFL rate of a loaded FP32-mixed stage: the point value from the average
@@ -670,7 +742,7 @@ __global__ void __launch_bounds__(256) stage_rate2d_mx(const float* planes, long
 #pragma unroll
             for (int qq = 1; qq < NQ; ++qq) d[qq] = planes[(long long)(v * NQ + qq) * plane + cell];
             const ff ub{planes[(long long)(v * NQ) * plane + cell], planes[(long long)(NV * NQ + v) * plane + cell]};
-            centre[v] = wcc::ff_add(ub, -even_correction<P>(d)).hi;
+            centre[v] = wcc::ff_add(ub, -even_correction<P, float>(d)).hi;
         }
         const float r = cfl_rate<SYS, float>(centre, law, (float)(1.0 / dx), (float)(1.0 / dy));
         if (r != r) {
@@ -680,14 +752,7 @@ __global__ void __launch_bounds__(256) stage_rate2d_mx(const float* planes, long
             m = r;
         }
     }
-    double r = (double)m;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) r = fmax(r, __shfl_xor_sync(0xffffffffu, r, o));
-    err = __reduce_or_sync(0xffffffffu, err);
-    if ((threadIdx.x & 31) == 0) {
-        atomicMax(&st->rate_bits[0], (unsigned long long)__double_as_longlong(r));
-        if (err) atomicOr(&st->err, err);
-    }
+    post_rate((double)m, err, st);
 }
 
 template <int SYS, int P>
@@ -707,8 +772,9 @@ namespace wcc2d {
 cudaError_t launch_halfstep2d_mx(int system, int P, const Step2D& a, cudaStream_t stream);
 cudaError_t launch_stage_rate2d_mx(int system, int P, const float* planes, long long pitch, long long plane, int nx,
                                    int ny, const Law2D& law, double dx, double dy, DevState2D* st, cudaStream_t stream);
-cudaError_t launch_convert2d_mx(int P, bool to_planes, double* aos, float* planes, int nx, int ny, int nv,
-                                long long pitch, long long plane, cudaStream_t stream);
+// precision: 0 FP64, 1 FP32, 2 FP32-mixed planes
+cudaError_t launch_convert2d(int P, int precision, bool to_planes, double* aos, void* planes, int nx, int ny, int nv,
+                             long long pitch, long long plane, cudaStream_t stream);
 }  // namespace wcc2d
 
 namespace wcc2d {

@@ -1,5 +1,5 @@
 // 2D FP32-mixed half-step kernels (advection, Burgers, Euler; P = 1..3), the
-// stage CFL rate and the layout conversions of the FP32-mixed storage.
+// stage CFL rate, and the layout conversions of every 2D storage.
 #include "wcc2d_kernels.cuh"
 
 namespace wcc2d {
@@ -56,27 +56,24 @@ cudaError_t launch_stage_rate2d_mx(int system, int P, const float* planes, long 
     }
 }
 
-cudaError_t launch_convert2d_mx(int P, bool to_planes, double* aos, float* planes, int nx, int ny, int nv,
-                                long long pitch, long long plane, cudaStream_t stream) {
-    const long long n = (long long)nx * ny;
-    const int grid = (int)std::min<long long>((n + 255) / 256, 152 * 16);
+namespace {
+template <bool MX, class T>
+cudaError_t convert_p(int P, bool to_planes, double* aos, void* planes, int nx, int ny, int nv, long long pitch,
+                      long long plane, cudaStream_t stream) {
     switch (P) {
-        case 1:
-            if (to_planes) aos_to_planes2d_mx<1><<<grid, 256, 0, stream>>>(aos, planes, nx, ny, nv, pitch, plane);
-            else planes_to_aos2d_mx<1><<<grid, 256, 0, stream>>>(planes, aos, nx, ny, nv, pitch, plane);
-            break;
-        case 2:
-            if (to_planes) aos_to_planes2d_mx<2><<<grid, 256, 0, stream>>>(aos, planes, nx, ny, nv, pitch, plane);
-            else planes_to_aos2d_mx<2><<<grid, 256, 0, stream>>>(planes, aos, nx, ny, nv, pitch, plane);
-            break;
-        case 3:
-            if (to_planes) aos_to_planes2d_mx<3><<<grid, 256, 0, stream>>>(aos, planes, nx, ny, nv, pitch, plane);
-            else planes_to_aos2d_mx<3><<<grid, 256, 0, stream>>>(planes, aos, nx, ny, nv, pitch, plane);
-            break;
-        default:
-            return cudaErrorInvalidValue;
+        case 1: return launch_convert2d_t<1, MX, T>(to_planes, aos, planes, nx, ny, nv, pitch, plane, stream);
+        case 2: return launch_convert2d_t<2, MX, T>(to_planes, aos, planes, nx, ny, nv, pitch, plane, stream);
+        case 3: return launch_convert2d_t<3, MX, T>(to_planes, aos, planes, nx, ny, nv, pitch, plane, stream);
+        default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t launch_convert2d(int P, int precision, bool to_planes, double* aos, void* planes, int nx, int ny, int nv,
+                             long long pitch, long long plane, cudaStream_t stream) {
+    if (precision == 2) return convert_p<true, float>(P, to_planes, aos, planes, nx, ny, nv, pitch, plane, stream);
+    if (precision == 1) return convert_p<false, float>(P, to_planes, aos, planes, nx, ny, nv, pitch, plane, stream);
+    return convert_p<false, double>(P, to_planes, aos, planes, nx, ny, nv, pitch, plane, stream);
 }
 
 }  // namespace wcc2d
