@@ -352,28 +352,38 @@ constexpr int mixed2_smem_float2() {
 // io.first_new + s - parity, through the boundary rule): the cell average
 // ub (float-float) and the Taylor coefficients c[v][1..P] (c[v][0] is left
 // for mixed_parent_records).
-template <int SYS, int P, bool COMP>
+// INNER: tiles whose parents all are cells of the stage take a path of their
+// own, where each plane's address is the same for the whole CTA up to the
+// thread's number (no 64-bit addition per access: 263 -> 253 us per half-step for
+// the batch of 768, 129.5 -> 127.9 us for 2^22 cells, Euler P = 3).  Scalar systems
+// (a third of the loads; Burgers P = 4 at 250 007 cells 7.7 -> 7.9 us with it) and the
+// cluster kernel, bound by the latency of one tile, do better with the shorter code.
+template <int SYS, int P, bool COMP, bool INNER = (SYS == EULER)>
 __device__ __forceinline__ void mixed_load_parents(const TileIO& io, ff2 (&ub)[nvars(SYS)],
                                                    f2 (&c)[nvars(SYS)][P + 1]) {
     constexpr int NV = nvars(SYS);
     constexpr int K = P + 1;
     constexpr int NP = P + 2;
-    const int t = threadIdx.x;
-    const long long base = io.first_new + t - (io.parity ? 1 : 0);
-    const long long pa = parent_index(base, io.n_old, io.bc);
-    const long long pb = parent_index(base + kThreadsMixed, io.n_old, io.bc);
-    sfor<0, NV>([&](auto V) {
-        constexpr int v = decltype(V)::value;
-        const float* p0 = io.in32 + (long long)(v * NP + 0) * io.pitch;
-        const float* p1 = io.in32 + (long long)(v * NP + 1) * io.pitch;
-        ub[v].hi = f2(p0[pa], p0[pb]);
-        ub[v].lo = COMP ? f2(p1[pa], p1[pb]) : f2(0.f);
-        sfor<1, K>([&](auto Ki) {
-            constexpr int k = decltype(Ki)::value;
-            const float* pk = io.in32 + (long long)(v * NP + k + 1) * io.pitch;
-            c[v][k] = f2(pk[pa], pk[pb]);
+    const unsigned t = threadIdx.x;
+    const long long first = io.first_new - (io.parity ? 1 : 0);  // parent of slot 0
+    auto load = [&](const float* tile, long long pitch, auto at) {
+        sfor<0, NV>([&](auto V) {
+            constexpr int v = decltype(V)::value;
+            ub[v].hi = at(tile + (v * NP + 0) * pitch);
+            ub[v].lo = COMP ? at(tile + (v * NP + 1) * pitch) : f2(0.f);
+            sfor<1, K>([&](auto Ki) {
+                constexpr int k = decltype(Ki)::value;
+                c[v][k] = at(tile + (v * NP + k + 1) * pitch);
+            });
         });
-    });
+    };
+    if (INNER && first >= 0 && first + 2 * kThreadsMixed <= io.n_old) {
+        load(io.in32 + first, io.pitch, [&](const float* p) { return f2(p[t], p[t + kThreadsMixed]); });
+    } else {
+        const long long pa = parent_index(first + t, io.n_old, io.bc);
+        const long long pb = parent_index(first + t + kThreadsMixed, io.n_old, io.bc);
+        load(io.in32, io.pitch, [&](const float* p) { return f2(p[pa], p[pb]); });
+    }
 }
 
 // Phase 1: the records of this thread's two parents (cell averages ub,
@@ -583,29 +593,23 @@ __device__ __forceinline__ float mixed_store(const TileIO& io, const ff2 (&ubn)[
     constexpr int NV = nvars(SYS);
     constexpr int K = P + 1;
     constexpr int NP = P + 2;
-    const long long ia = io.first_new + threadIdx.x;
-    const long long ib = ia + kThreadsMixed;
+    const unsigned t = threadIdx.x;
+    float* tile = io.out32 + io.first_new;
     f2 u0n[NV];
     f2 check(0.f);  // NaN / Inf in any stored value reaches this sum
+    auto store = [&](float* p, f2 x) {
+        if (va) __stcs(p + t, x.x());
+        if (vb) __stcs(p + t + kThreadsMixed, x.y());
+    };
     sfor<0, NV>([&](auto V) {
         constexpr int v = decltype(V)::value;
         check += ubn[v].hi;
-        float* o0 = io.out32 + (long long)(v * NP + 0) * io.pitch;
-        float* o1 = io.out32 + (long long)(v * NP + 1) * io.pitch;
-        if (va) {
-            __stcs(o0 + ia, ubn[v].hi.x());
-            __stcs(o1 + ia, ubn[v].lo.x());
-        }
-        if (vb) {
-            __stcs(o0 + ib, ubn[v].hi.y());
-            __stcs(o1 + ib, ubn[v].lo.y());
-        }
+        store(tile + (v * NP + 0) * io.pitch, ubn[v].hi);
+        store(tile + (v * NP + 1) * io.pitch, ubn[v].lo);
         sfor<1, K>([&](auto Ki) {
             constexpr int k = decltype(Ki)::value;
             check += d[v][k];
-            float* ok = io.out32 + (long long)(v * NP + k + 1) * io.pitch;
-            if (va) __stcs(ok + ia, d[v][k].x());
-            if (vb) __stcs(ok + ib, d[v][k].y());
+            store(tile + (v * NP + k + 1) * io.pitch, d[v][k]);
         });
         u0n[v] = ubn[v].hi + d[v][0];
     });
@@ -623,7 +627,7 @@ __device__ __forceinline__ float mixed_store(const TileIO& io, const ff2 (&ubn)[
 // half-step's size; it is called after the parents' loads have been issued,
 // so that reading the device state does not delay them (the state's fields
 // decide a branch, which waits for them).
-template <int SYS, int P, bool COMP, bool PARK = (P >= 3), class Step>
+template <int SYS, int P, bool COMP, bool PARK = (P >= 3), bool INNER = (SYS == EULER), class Step>
 __device__ __forceinline__ void mixed_tile2(const TileIO& io, Step&& step, const StepArgs& args, float2* rec,
                                             float& speed, unsigned& err) {
     constexpr int NV = nvars(SYS);
@@ -632,7 +636,7 @@ __device__ __forceinline__ void mixed_tile2(const TileIO& io, Step&& step, const
     {
         ff2 ub[NV];
         f2 c[NV][K];
-        mixed_load_parents<SYS, P, COMP>(io, ub, c);
+        mixed_load_parents<SYS, P, COMP, INNER>(io, ub, c);
         const StepSize& z = step();
         const ff2 lam2{f2(z.lam_hi), f2(COMP ? z.lam_lo : 0.f)};
         mixed_parent_records<SYS, P, COMP, PARK>(ub, c, lam2, args, rec);
