@@ -537,8 +537,13 @@ __device__ __forceinline__ void first_derivatives(R (&d)[nq(P)], const R (&vv)[4
 // The odd terms drop out of their means:
 //   r_0 = r_2 = a + e_11 / 4 - (v_0 + v_2) / 2,  r_1 = r_3 = a - e_11 / 4 - (v_1 + v_3) / 2,
 // a = (e_20 + e_02) (1/4 - 1/12) the even part at a vertex less the average.
+//
+// Returns false, with d as it was, where the limiter does not act: FP64 with
+// sigma tau below 2^-31 of every denominator (compared on the exponents), FP32
+// below 2^-15 of them (the side weights, squares of the ratios, are then below
+// 2^-62 and 2^-30: w_0 is 1).
 template <int P, class R>
-__device__ __forceinline__ void limit_scalar(R (&d)[nq(P)], const R (&vv)[4], const Law2D& law, R ub) {
+__device__ __forceinline__ bool limit_scalar(R (&d)[nq(P)], const R (&vv)[4], const Law2D& law, R ub) {
     constexpr int NQ = nq(P);
     R sx[5], sy[5];
     sx[1] = -(vv[0] + vv[3]);
@@ -620,8 +625,16 @@ __device__ __forceinline__ void limit_scalar(R (&d)[nq(P)], const R (&vv)[4], co
         }
         const R st = (half_sigma + half_sigma) * tau;
         if constexpr (!is_f32<R>) {
+            R den[5];
+            int least = 2047;
 #pragma unroll
-            for (int m = 0; m < 5; ++m) w[m] = weight_pow(st * recip_t(fma(beta[m], beta[m], eps)), law);
+            for (int m = 0; m < 5; ++m) {
+                den[m] = fma(beta[m], beta[m], eps);
+                least = min(least, wcc::exponent_of(den[m]));
+            }
+            if (law.alpha_is_two && wcc::exponent_of(st) + 32 <= least) return false;
+#pragma unroll
+            for (int m = 0; m < 5; ++m) w[m] = weight_pow(st * recip_t(den[m]), law);
             const R rest = (w[1] + w[2]) + (w[3] + w[4]);
             const R is = recip_t((w[0] + cst<R>(1.0)) + rest);
 #pragma unroll
@@ -636,6 +649,7 @@ __device__ __forceinline__ void limit_scalar(R (&d)[nq(P)], const R (&vv)[4], co
                 den[m] = fmaf(beta[m], beta[m], eps);
                 dmin = fminf(dmin, den[m]);
             }
+            if (law.alpha_is_two && !(st * 0x1p15f >= dmin)) return false;
             // the "1 +" of w_0, rescaled.  dmin and st both scaled by 2^64
             // (exact), so that a subnormal st (its dmin can be subnormal too:
             // eps = 1e-40) is a normal number for the reciprocal; st above
@@ -672,6 +686,7 @@ __device__ __forceinline__ void limit_scalar(R (&d)[nq(P)], const R (&vv)[4], co
     d[2] = l2;
 #pragma unroll
     for (int i = 3; i < NQ; ++i) d[i] = w[0] * d[i];
+    return true;
 }
 
 // Rotated characteristic limiting for the 2D Euler equations (Sec. 4):
@@ -740,10 +755,16 @@ __device__ __forceinline__ bool limit_euler(R (&D)[4][nq(P)], const R (&ub)[4], 
 #pragma unroll
             for (int i = 0; i < 4; ++i) cd[i][qq] = w[i];
         }
+        bool limited = false;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             first_derivatives<P>(cd[i], cvv[i]);
-            limit_scalar<P>(cd[i], cvv[i], law, cub[i]);
+            limited |= limit_scalar<P>(cd[i], cvv[i], law, cub[i]);
+        }
+        if (!limited) {  // nothing to map back
+#pragma unroll
+            for (int j = 0; j < 4; ++j) first_derivatives<P>(D[j], vv[j]);
+            return true;
         }
 #pragma unroll
         for (int qq = 1; qq < NQ; ++qq) {

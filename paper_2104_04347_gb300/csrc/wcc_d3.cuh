@@ -62,6 +62,9 @@ __device__ __forceinline__ bool all_pos(d3 a) {
 // NaN / Inf test on the exponent bits
 __device__ __forceinline__ bool not_finite(d3 x) { return (__double2hiint(x.v) & 0x7ff00000) == 0x7ff00000; }
 
+// Exponent field (0: zero or subnormal, 2047: infinity or NaN).
+__device__ __forceinline__ int exponent_of(d3 a) { return (int)(((unsigned)__double2hiint(a.v) >> 20) & 0x7ffu); }
+
 // Exponent between 2^-1000 and 2^1000: where the estimates below are normal
 // and their residuals exact to rounding.  Everything else (zeros, infinities,
 // NaN, extreme values, negative roots) takes the compiler's operations.

@@ -241,15 +241,14 @@ __device__ __forceinline__ void fp64_tile(const TileIO64& io, Step&& step, const
             high_derivatives<P, d3>(vL, vR, e[v]);
         });
 
-        if (!args.limiter) {
-            sfor<0, NV>([&](auto V) {
-                constexpr int v = decltype(V)::value;
-                e[v][1] = first_derivative<P, d3>(e[v], dl[v], dr[v]);
-            });
-        } else if constexpr (NV == 1) {
+        bool limited = false;
+        if constexpr (NV == 1) {
             e[0][1] = first_derivative<P, d3>(e[0], dl[0], dr[0]);
-            limit_deviation<P, d3>(e[0], dl[0], dr[0], args);
-        } else {
+            if (args.limiter) {
+                LimiterTerms<d3> T;
+                if (limiter_terms<P, d3>(e[0], dl[0], dr[0], args, T)) apply_limiter<P, d3>(e[0], T, args);
+            }
+        } else if (args.limiter) {
             // Sec. 4: limit characteristic variables L(ubar) U, map back with
             // R(ubar).  e_1 is linear in the differences and the higher
             // coefficients, so it is formed after the projection.
@@ -269,11 +268,23 @@ __device__ __forceinline__ void fp64_tile(const TileIO64& io, Step&& step, const
             sfor<0, 3>([&](auto Ii) {
                 constexpr int r = decltype(Ii)::value;
                 ce[r][1] = first_derivative<P, d3>(ce[r], cdl[r], cdr[r]);
-                limit_deviation<P, d3>(ce[r], cdl[r], cdr[r], args);
+                LimiterTerms<d3> T;
+                if (limiter_terms<P, d3>(ce[r], cdl[r], cdr[r], args, T)) {
+                    apply_limiter<P, d3>(ce[r], T, args);
+                    limited = true;
+                }
             });
-            sfor<1, K>([&](auto Ki) {
-                constexpr int k = decltype(Ki)::value;
-                E.right(ce[0][k], ce[1][k], ce[2][k], e[0][k], e[1][k], e[2][k]);
+            if (limited) {
+                sfor<1, K>([&](auto Ki) {
+                    constexpr int k = decltype(Ki)::value;
+                    E.right(ce[0][k], ce[1][k], ce[2][k], e[0][k], e[1][k], e[2][k]);
+                });
+            }
+        }
+        if (NV > 1 && !limited) {
+            sfor<0, NV>([&](auto V) {
+                constexpr int v = decltype(V)::value;
+                e[v][1] = first_derivative<P, d3>(e[v], dl[v], dr[v]);
             });
         }
         sfor<0, NV>([&](auto V) {  // the limiter keeps the cell average
