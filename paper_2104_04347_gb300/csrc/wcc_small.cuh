@@ -82,19 +82,25 @@ __global__ void __launch_bounds__(kThreadsMixed) halfstep_small(const StepArgs a
     StepSize z;
     int s = 0;
     // the bound of the stage that half-step s - 1 made
-    auto bound = [&]() -> double {
+    auto bound_key = [&]() -> Key {
         Key k = keys[(s - 1) & 1][lane];
         const Key k2 = keys[(s - 1) & 1][lane + 32];
-        k = warp_max_key(k2 > k ? k2 : k);
+        return warp_max_key(k2 > k ? k2 : k);
+    };
+    auto value = [](Key k) -> double {
         if constexpr (F32) return (double)__uint_as_float(k);
         else return __longlong_as_double((long long)k);
     };
+    Key sized_key = 0;  // the bound that z's quotients were taken from (none at first)
     int sized = -1;  // the half-step that z belongs to
     auto step = [&]() -> const StepSize& {
         if (sized == s) return z;
         sized = s;
         if (s == 0) return z = step_size(args);
-        cfl_quotients(args.cfl, args.dx, args.inv_dx, bound(), z.dt, z.lam);
+        const Key k = bound_key();
+        if (k == sized_key) return z;  // waves of constant speed keep their half-step
+        sized_key = k;
+        cfl_quotients(args.cfl, args.dx, args.inv_dx, value(k), z.dt, z.lam);
         if constexpr (F32) split_to_floats(z.lam, z.lam_hi, z.lam_lo);
         return z;
     };
@@ -136,7 +142,7 @@ __global__ void __launch_bounds__(kThreadsMixed) halfstep_small(const StepArgs a
     err = __reduce_or_sync(0xffffffffu, err);
     if (lane == 0 && err) atomicOr(&st->err, err);
     if (s == 0) return;  // nothing fitted: the state is as it was
-    const double amax = bound();
+    const double amax = value(bound_key());
     if (keeper) {
         // what the last single half-step's bookkeeping would leave
         const int now = args.parity ^ (s & 1);
