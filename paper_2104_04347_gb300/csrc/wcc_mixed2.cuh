@@ -239,24 +239,34 @@ __device__ __forceinline__ f2 scaled_eps(const StepArgs& args) {
     return f2(fmaxf(args.eps_f, 1.4e-45f) * 4294967296.f);
 }
 
+// d_m 2^32 of the weights for P >= 2, and the least of them.
+__device__ __forceinline__ f2 scaled_denominators(f2 b0, f2 b1, f2 b2, const StepArgs& args, f2& d0, f2& d1, f2& d2) {
+    const f2 eps = scaled_eps(args), s16(65536.f);
+    const f2 c0 = b0 * s16, c1 = b1 * s16, c2 = b2 * s16;
+    d0 = fma(c0, c0, eps);
+    d1 = fma(c1, c1, eps);
+    d2 = fma(c2, c2, eps);
+    return fmin(d0, fmin(d1, d2));
+}
+
+// With st below 2^-30 of every denominator in both cells the limiter does not
+// act: w_0 rounds to 1 and w_1, w_2 are below 2^-60.
+__device__ __forceinline__ bool limiter_acts_f2(f2 b0, f2 b1, f2 b2, f2 st, const StepArgs& args) {
+    f2 d0, d1, d2;
+    const f2 dmin = scaled_denominators(b0, b1, b2, args, d0, d1, d2), far = st * f2(0x1p62f);
+    return !(args.alpha_is_two && far.x() < dmin.x() && far.y() < dmin.y());
+}
+
 // Normalised weights for P >= 2 (Eq. 1DHighOrderWeights), scale-free:
 // w0 ~ 1 + (st/d0)^alpha, w_m ~ (st/d_m)^alpha with d = beta^2 + eps, all
 // multiplied through by (d_min/st)^alpha, so every ratio is at most 1 (st = 0
 // makes the first ratio +inf, clamped to 1e18).  w0 is formed as 1 - w1 - w2
 // so that it is exactly 1 whenever the other two vanish.
-// With st below 2^-30 d_min in both cells the limiter does not act: w_0 rounds to 1
-// and w_1, w_2 are below 2^-60.  Then the function returns false without forming
-// them (eight reciprocal estimates and some thirty other instructions: Euler P = 3
-// at 2^22 cells 127.5 -> 122.9 us per half-step, two half-steps per launch at P = 2
-// 24.7 -> 23.0 us).
-__device__ __forceinline__ bool weights_hi_f2(f2 b0, f2 b1, f2 b2, f2 st, const StepArgs& args, f2& w0, f2& w1,
+__device__ __forceinline__ void weights_hi_f2(f2 b0, f2 b1, f2 b2, f2 st, const StepArgs& args, f2& w0, f2& w1,
                                               f2& w2) {
-    const f2 eps = scaled_eps(args), s16(65536.f), s32(4294967296.f);
-    const f2 c0 = b0 * s16, c1 = b1 * s16, c2 = b2 * s16;
-    const f2 d0 = fma(c0, c0, eps), d1 = fma(c1, c1, eps), d2 = fma(c2, c2, eps);  // d 2^32
-    const f2 dmin = fmin(d0, fmin(d1, d2));
-    const f2 far = st * f2(0x1p62f);
-    if (args.alpha_is_two && far.x() < dmin.x() && far.y() < dmin.y()) return false;
+    f2 d0, d1, d2;
+    const f2 dmin = scaled_denominators(b0, b1, b2, args, d0, d1, d2);
+    const f2 s32(4294967296.f);
     const f2 q0 = dmin * rcp_est(d0), q1 = dmin * rcp_est(d1), q2 = dmin * rcp_est(d2);
     const f2 z = fmin(dmin * rcp_est(st * s32), f2(1e18f));  // st = 0 gives +inf -> 1e18
     f2 h0, h1, h2;
@@ -274,7 +284,6 @@ __device__ __forceinline__ bool weights_hi_f2(f2 b0, f2 b1, f2 b2, f2 st, const 
     w1 = h1 * inv;
     w2 = h2 * inv;
     w0 = f2(1.f) - (w1 + w2);
-    return true;
 }
 
 // Normalised weights for P = 1 (Eq. 1D2ndOrderWeights): w_m proportional to
@@ -301,13 +310,10 @@ __device__ __forceinline__ void weights_p1_f2(f2 b0, f2 b1, f2 b2, const StepArg
     w0 = f2(1.f) - (w1 + w2);
 }
 
-// Limiter of Sec. 2.2 in deviation form, paired.  d[0] = u_0(centre) - ubar,
-// d[1..P] = Taylor coefficients; dl = ubar - u_{i-1/2}, dr = u_{i+1/2} - ubar.
-// On return d holds the same quantities of the limited polynomial.
+// beta_m and (P >= 2) sigma tau of the limiter, paired; arguments as below.
 template <int P>
-__device__ __forceinline__ void limit_deviation_f2(f2 (&d)[P + 1], f2 dl, f2 dr, const StepArgs& args) {
+__device__ __forceinline__ f2 limiter_betas_f2(const f2 (&d)[P + 1], f2 dl, f2 dr, f2& b0, f2& b1, f2& b2) {
     const f2 s1 = f2(2.f) * dl, s2 = f2(2.f) * dr;
-    f2 b0;
     sfor<1, P + 1>([&](auto Ji) {
         constexpr int j = decltype(Ji)::value;
         f2 row = times<csmooth(j, j) == 1.0>(d[j], csmooth(j, j));
@@ -319,10 +325,10 @@ __device__ __forceinline__ void limit_deviation_f2(f2 (&d)[P + 1], f2 dl, f2 dr,
         if constexpr (j == 1) b0 = row * d[1];
         else b0 = fma(row, d[j], b0);
     });
-    const f2 b1 = s1 * s1, b2 = s2 * s2;
-    f2 w0, w1, w2;
+    b1 = s1 * s1;
+    b2 = s2 * s2;
     if constexpr (P == 1) {
-        weights_p1_f2(b0, b1, b2, args, w0, w1, w2);
+        return f2(0.f);
     } else {
         f2 up = d[0], um = d[0];
         sfor<1, P + 1>([&](auto Ki) {
@@ -334,8 +340,37 @@ __device__ __forceinline__ void limit_deviation_f2(f2 (&d)[P + 1], f2 dl, f2 dr,
         const f2 rl = um + dl;
         const f2 sigma = fma(rr, rr, rl * rl);
         const f2 tp = f2((float)cfact(P)) * d[P];
-        if (!weights_hi_f2(b0, b1, b2, sigma * (tp * tp), args, w0, w1, w2)) return;
+        return sigma * (tp * tp);
     }
+}
+
+// Whether the limiter acts on the component in either cell (always for P = 1).
+template <int P>
+__device__ __forceinline__ bool limiter_acts_f2(const f2 (&d)[P + 1], f2 dl, f2 dr, const StepArgs& args) {
+    if constexpr (P == 1) return true;
+    f2 b0, b1, b2;
+    const f2 st = limiter_betas_f2<P>(d, dl, dr, b0, b1, b2);
+    return limiter_acts_f2(b0, b1, b2, st, args);
+}
+
+// Limiter of Sec. 2.2 in deviation form, paired.  d[0] = u_0(centre) - ubar,
+// d[1..P] = Taylor coefficients; dl = ubar - u_{i-1/2}, dr = u_{i+1/2} - ubar.
+// On return d holds the same quantities of the limited polynomial.  ASK: first
+// see whether the limiter acts, and leave the weights (eight reciprocal
+// estimates and some thirty other instructions) out where it does not: Euler
+// P = 3 at 2^22 cells 127.5 -> 122.9 us per half-step, two half-steps per launch at
+// P = 2 24.7 -> 23.0 us.
+template <int P, bool ASK = true>
+__device__ __forceinline__ void limit_deviation_f2(f2 (&d)[P + 1], f2 dl, f2 dr, const StepArgs& args) {
+    f2 b0, b1, b2, w0, w1, w2;
+    const f2 st = limiter_betas_f2<P>(d, dl, dr, b0, b1, b2);
+    if constexpr (P == 1) {
+        weights_p1_f2(b0, b1, b2, args, w0, w1, w2);
+    } else {
+        if (ASK && !limiter_acts_f2(b0, b1, b2, st, args)) return;
+        weights_hi_f2(b0, b1, b2, st, args, w0, w1, w2);
+    }
+    const f2 s1 = f2(2.f) * dl, s2 = f2(2.f) * dr;
     d[0] *= w0;
     d[1] = fma(w0, d[1], fma(w1, s1, w2 * s2));
     sfor<2, P + 1>([&](auto Ki) { d[decltype(Ki)::value] *= w0; });
@@ -507,7 +542,10 @@ __device__ __forceinline__ void mixed_parent_records(const ff2 (&ub_in)[nvars(SY
 // records of slots (t, t + 1) and (t + kThreadsMixed, t + kThreadsMixed + 1):
 // the cell average ubn (float-float), the point value minus the average
 // d[v][0] and the coefficients d[v][1..P] of the limited polynomial.
-template <int SYS, int P, bool COMP>
+// SMALL: for a mesh of one tile per SM, where a warp has its scheduler to itself
+// and the three components' chains should stay side by side: one question for
+// all three (it holds more registers than the large meshes' occupancy allows).
+template <int SYS, int P, bool COMP, bool SMALL = false>
 __device__ __forceinline__ void mixed_new_cells(const float2* rec, const StepArgs& args, ff2 (&ubn)[nvars(SYS)],
                                                 f2 (&d)[nvars(SYS)][P + 1], unsigned& err) {
     using A = FF<COMP>;
@@ -564,11 +602,22 @@ __device__ __forceinline__ void mixed_new_cells(const float2* rec, const StepArg
                 cd[1][k] = w[1];
                 cd[2][k] = w[2];
             });
-            sfor<0, 3>([&](auto Ii) {
-                constexpr int rr = decltype(Ii)::value;
-                cd[rr][0] = -average_minus_centre<P>(cd[rr]);
-                limit_deviation_f2<P>(cd[rr], cdl[rr], cdr[rr], args);
-            });
+            bool acts = true;
+            if constexpr (SMALL) {
+                acts = false;
+                sfor<0, 3>([&](auto Ii) {
+                    constexpr int rr = decltype(Ii)::value;
+                    cd[rr][0] = -average_minus_centre<P>(cd[rr]);
+                    acts |= limiter_acts_f2<P>(cd[rr], cdl[rr], cdr[rr], args);
+                });
+            }
+            if (acts) {
+                sfor<0, 3>([&](auto Ii) {
+                    constexpr int rr = decltype(Ii)::value;
+                    cd[rr][0] = -average_minus_centre<P>(cd[rr]);
+                    limit_deviation_f2<P, !SMALL>(cd[rr], cdl[rr], cdr[rr], args);
+                });
+            }
             sfor<1, K>([&](auto Ki) {
                 constexpr int k = decltype(Ki)::value;
                 E.right(cd[0][k], cd[1][k], cd[2][k], d[0][k], d[1][k], d[2][k]);
@@ -636,7 +685,7 @@ __device__ __forceinline__ float mixed_store(const TileIO& io, const ff2 (&ubn)[
 // half-step's size; it is called after the parents' loads have been issued,
 // so that reading the device state does not delay them (the state's fields
 // decide a branch, which waits for them).
-template <int SYS, int P, bool COMP, bool PARK = (P >= 3), bool INNER = (SYS == EULER), class Step>
+template <int SYS, int P, bool COMP, bool PARK = (P >= 3), bool SMALL = false, class Step>
 __device__ __forceinline__ void mixed_tile2(const TileIO& io, Step&& step, const StepArgs& args, float2* rec,
                                             float& speed, unsigned& err) {
     constexpr int NV = nvars(SYS);
@@ -645,7 +694,7 @@ __device__ __forceinline__ void mixed_tile2(const TileIO& io, Step&& step, const
     {
         ff2 ub[NV];
         f2 c[NV][K];
-        mixed_load_parents<SYS, P, COMP, INNER>(io, ub, c);
+        mixed_load_parents<SYS, P, COMP, SYS == EULER && !SMALL>(io, ub, c);
         const StepSize& z = step();
         const ff2 lam2{f2(z.lam_hi), f2(COMP ? z.lam_lo : 0.f)};
         mixed_parent_records<SYS, P, COMP, PARK>(ub, c, lam2, args, rec);
@@ -653,7 +702,7 @@ __device__ __forceinline__ void mixed_tile2(const TileIO& io, Step&& step, const
     __syncthreads();
     ff2 ubn[NV];
     f2 d[NV][K];
-    mixed_new_cells<SYS, P, COMP>(rec, args, ubn, d, err);
+    mixed_new_cells<SYS, P, COMP, SMALL>(rec, args, ubn, d, err);
     const long long ia = io.first_new + t;
     const bool va = ia < io.n_new;
     const bool vb = (t < kThreadsMixed - 1) && ia + kThreadsMixed < io.n_new;

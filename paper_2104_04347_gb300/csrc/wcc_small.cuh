@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(kThreadsMixed) halfstep_small(const StepArgs a
             const TileIO io{odd ? args.out32 : args.in32, odd ? const_cast<float*>(args.in32) : args.out32, args.pitch,
                             n_old, n_new, (long long)rank * kTileCells, parity, args.bc};
             float speed = 0.f;
-            mixed_tile2<SYS, P, true, (P >= 3), false>(io, step, args, rec32, speed, err);
+            mixed_tile2<SYS, P, true, (P >= 3), true>(io, step, args, rec32, speed, err);
             if (speed != speed) {
                 speed = INFINITY;
                 err |= ERR_NONFINITE;
