@@ -57,7 +57,8 @@ __global__ void __launch_bounds__(kThreadsMixed, (mixed_min_ctas<PA>() < mixed_m
     constexpr int SB = mixed2_smem_float2<SYS, PB>();
     __shared__ float2 rec[SA > SB ? SA : SB];
     pdl_begin();
-    for (long long tile = blockIdx.x; tile < b.total_tiles; tile += LOOP ? (long long)gridDim.x : b.total_tiles) {
+    for (long long n = blockIdx.x; n < b.total_tiles; n += LOOP ? (long long)gridDim.x : b.total_tiles) {
+        const long long tile = sweep_index<SYS == EULER>(b.in[0], b.out[0], n, b.total_tiles);
         const int i = __ldg(b.tile_inst + tile);
         const BatchInstance& I = b.inst[i];
         DevState* st = b.st + i;
@@ -97,7 +98,8 @@ __global__ void __launch_bounds__(kThreadsMixed, (mixed_min_ctas<PA>() < mixed_m
     __shared__ float2 rec[SA > SB ? SA : SB];
     pdl_begin();
     const unsigned refused = *(volatile unsigned*)b.tb_refused;
-    for (long long tile = blockIdx.x; tile < b.total_tiles; tile += LOOP ? (long long)gridDim.x : b.total_tiles) {
+    for (long long n = blockIdx.x; n < b.total_tiles; n += LOOP ? (long long)gridDim.x : b.total_tiles) {
+        const long long tile = sweep_index<SYS == EULER>(b.in[0], b.out[0], n, b.total_tiles);
         const int i = __ldg(b.tile_inst + tile);
         const BatchInstance& I = b.inst[i];
         DevState* st = b.st + i;

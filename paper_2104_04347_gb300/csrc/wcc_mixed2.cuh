@@ -422,11 +422,11 @@ __device__ __forceinline__ void mixed_load_parents(const TileIO& io, ff2 (&ub)[n
         });
     };
     if (INNER && first >= 0 && first + 2 * kThreadsMixed <= io.n_old) {
-        load(io.in32 + first, io.pitch, [&](const float* p) { return f2(p[t], p[t + kThreadsMixed]); });
+        load(io.in32 + first, io.pitch, [&](const float* p) { return f2(load_once<SYS == EULER>(p + t), load_once<SYS == EULER>(p + t + kThreadsMixed)); });
     } else {
         const long long pa = parent_index(first + t, io.n_old, io.bc);
         const long long pb = parent_index(first + t + kThreadsMixed, io.n_old, io.bc);
-        load(io.in32, io.pitch, [&](const float* p) { return f2(p[pa], p[pb]); });
+        load(io.in32, io.pitch, [&](const float* p) { return f2(load_once<SYS == EULER>(p + pa), load_once<SYS == EULER>(p + pb)); });
     }
 }
 
@@ -720,12 +720,12 @@ __global__ void __launch_bounds__(kThreadsMixed, mixed_min_ctas<P>()) halfstep_m
     unsigned err = 0u;
     if constexpr (TPC == 1) {
         const TileIO io{args.in32, args.out32, args.pitch, args.n_old, args.n_new,
-                        (long long)blockIdx.x * kTileMixed, args.parity, args.bc};
+                        sweep_index<SYS == EULER>(args.in32, args.out32, blockIdx.x, gridDim.x) * kTileMixed, args.parity, args.bc};
         mixed_tile2<SYS, P, COMP>(io, [&]() -> const StepSize& { return z = step_size(args); }, args, rec, speed, err);
     } else {
         const long long ntiles = (args.n_new + kTileMixed - 1) / kTileMixed;
         for (int r = 0; r < TPC; ++r) {
-            const long long tile = (long long)blockIdx.x * TPC + r;
+            const long long tile = sweep_index<SYS == EULER>(args.in32, args.out32, blockIdx.x, gridDim.x) * TPC + r;
             if (tile >= ntiles) break;
             if (r) __syncthreads();  // the previous tile's records are read
             const TileIO io{args.in32, args.out32, args.pitch, args.n_old, args.n_new,
@@ -992,7 +992,7 @@ __global__ void __launch_bounds__(kThreadsMixed, mixed_min_ctas<P>()) halfstep_m
     if (args.st->err & ERR_CFL) return;  // an earlier pair was refused: the caller steps singly from there
     StepSize z;
     const PairIO io{args.in32, args.out32, args.pitch, args.n_old, args.n_mid, args.n_new,
-                    (long long)blockIdx.x * kTileTB, args.parity, args.bc};
+                    sweep_index<SYS == EULER>(args.in32, args.out32, blockIdx.x, gridDim.x) * kTileTB, args.parity, args.bc};
     float mid = 0.f, fin = 0.f;
     unsigned err = 0u;
     mixed_pair_tile<SYS, P, COMP>(io, [&]() -> const StepSize& { return z = step_size(args); }, args, rec, mid, fin, err);
