@@ -156,26 +156,26 @@ def peaks():
 # FP64 operations the half-step kernel issues per cell-update (Euler, P = 3,
 # limiter on), counted from the executed DADD / DMUL / DFMA instructions (ncu
 # smsp__sass_thread_inst_executed_op_d{add,mul,fma}_pred_on.sum over one
-# launch at N = 2^21, DFMA counted as 2) divided by the cells of the launch:
-# (2 x 692675342 + 306816515 + 163894018) / 2097152.5.
-FP64_FLOPS_PER_CELL_UPDATE = 885.04
+# launch at N = 2^20, DFMA counted as 2) divided by the cells of the launch.
+# Every operation is a three-register DFMA, additions and multiplications
+# too, so the figure measures the pipe's occupancy, not useful operations; the
+# limiter is left out where it does not act, most of this workload's cells.
+FP64_FLOPS_PER_CELL_UPDATE = (2 * 403418745 + 2105473) / 1048576.5
 # DRAM bytes (read + write) of one launch at the bench size (N = 2^22), from
 # one ncu capture each (dram__bytes_read.sum + dram__bytes_write.sum, one
 # launch after three warm-up launches of the same kernel, graphs of 32
 # half-steps; profiles/halfstep_mixed_euler_p3.md).  The writes of the last
 # tiles are still in L2 when the kernel ends, so the figure is a little below
 # the algorithmic one read + one write of the state.
-FP64_TRAFFIC_2_22 = 402869760 + 352474368
-MIXED_TRAFFIC_2_22 = 251716864 + 200629504
+FP64_TRAFFIC_2_22 = 402913792 + 347655168
+MIXED_TRAFFIC_2_22 = 251732736 + 199964416
 # FP32 flops per cell-update of the same kernel, from one capture at
-# N = 2^21 of its executed paired instructions (sm__sass_thread_inst_executed_
-# op_f{add2,ffma2,fmul2}, thread instructions over the 2097152.5 cells):
-# 135.0 FADD2, 143.6 FFMA2 and 82.3 FMUL2 per cell-update, plus 8.5 scalar
-# FMUL.  A thread carries two cells and a paired instruction does one
-# operation for each, so per cell-update that is 2 x 135.0 adds, 2 x 143.6
-# FMAs (2 flops each), 2 x 82.3 multiplies and 8.5 multiplies.  Lane-wise
-# min/max and compares are not counted.
-MIXED_FP32_FLOPS_PER_CELL = 270.0 + 2 * 287.2 + 164.6 + 8.5
+# N = 2^20 of its executed paired and scalar instructions
+# (sm__sass_thread_inst_executed_op_f{add2,ffma2,fmul2}, smsp__..._f{add,mul}):
+# a thread carries two cells and a paired instruction does one operation for
+# each.  Lane-wise min/max and compares are not counted; nor is the limiter's
+# blend where it does not act.
+MIXED_FP32_FLOPS_PER_CELL = (2 * 132668976 + 4 * 137933604 + 2 * 69493404 + 3158784 + 8949888) / 1048576.5
 # FP64 pipe peak of the GB300 (dense, nominal): 1.25 TFLOP/s.
 FP64_PEAK_TFLOPS = 1.25
 
@@ -799,17 +799,19 @@ BYTES_2D_PER_CELL = {"fp32_mixed": 2 * 44 * 4, "fp32": 2 * 40 * 4, "fp64": 2 * 4
 # kernel, 64-thread strips) thread instructions of one launch at n = 1024
 # divided by the 1024^2 cells (FMA = 2 flops; min/max, compares and
 # conversions not counted; a paired FADD2 counts 2, a paired FFMA2 4).
-# FP32-mixed: its current kernel (96-thread strips, 19 rows per strip).
-# FP32: none, not recounted since its projections went to paired FP32.
-FLOPS_2D_PER_CELL = {"fp32_mixed": (1403120218 + 2 * 1618423496 + 264650802 + 2 * 12582912 + 4 * 155189248) / 1048576.0,
-                     "fp32": None,
-                     "fp64": (412078081 + 2 * 2396458776 + 341564899) / 1048576.0}
+# FP32-mixed: 96-thread strips.  FP64: every operation is a DFMA, so its figure
+# is the pipe's occupancy.
+FLOPS_2D_PER_CELL = {"fp32_mixed": (1205938660 + 2 * 1043579606 + 424629952 + 2 * 12582912 + 4 * 155189248) / 1048576.0,
+                     "fp32": (318283312 + 2 * 636306416 + 315836868 + 2 * 12582912 + 4 * 453492736 + 2 * 28827648) / 1048576.0,
+                     "fp64": 2 * 1967884767 / 1048576.0}
 # DRAM bytes (read + write) of one launch per cell, same captures; scaled by
 # cells to the bench size.  The writes undercount the stored DOFs: part of
 # the output is still in L2 when the kernel ends.  FP32-mixed: one launch at
 # the bench size itself, 2048^2, per strip height (a strip re-reads one parent
 # row, so the bytes depend slightly on it); heights not captured report none.
-TRAFFIC_2D_MIXED_BY_ROWS = {19: (780613888 + 691828736) / 4194304.0}
+# (for heights other than the default, 16, which stands for the picked one: 19
+# rows, measured before the Taylor form, the same planes)
+TRAFFIC_2D_MIXED_BY_ROWS = {16: (770688768 + 688579328) / 4194304.0, 19: (780613888 + 691828736) / 4194304.0}
 TRAFFIC_2D_PER_CELL = {"fp32_mixed": None, "fp32": None,
                        "fp64": (358728448 + 294830336) / 1048576.0}
 
@@ -916,11 +918,11 @@ CFL_HIGH = {3: 0.2, 4: 0.2, 5: 0.16, 6: 0.14}
 # FP64 flops per cell-update of halfstep_fp64<EULER, P> (ncu DADD + DMUL +
 # 2 DFMA thread instructions of one launch over the launch's cells); P = 3 is
 # FP64_FLOPS_PER_CELL_UPDATE, P = 4..6 from one launch each at N = 2^20
-# (e.g. P = 6: (132561538 + 271580931 + 2 x 1108567950) / 1048576.5).
+# (every operation a DFMA: the pipe's occupancy).
 FP64_FLOPS_HIGH = {3: None,
-                   4: (101969794 + 187162371 + 2 * 522598030) / 1048576.5,
-                   5: (120968962 + 232542339 + 2 * 766449806) / 1048576.5,
-                   6: (132561538 + 271580931 + 2 * 1108567950) / 1048576.5}
+                   4: (2105473 + 2 * 605019685) / 1048576.5,
+                   5: (2105473 + 2 * 884805957) / 1048576.5,
+                   6: (2105473 + 2 * 1271313777) / 1048576.5}
 
 
 def high_order_bench(args):
@@ -991,8 +993,9 @@ ORACLE_FLOPS = {(1, 1): 93.0, (1, 2): 191.0, (1, 3): 314.0, (1, 4): 502.0,
 # FP64 operations per cell-update the Burgers FP64 kernel executes
 # (halfstep_fp64<BURGERS, P>, limiter on): DADD + DMUL + 2 DFMA thread
 # instructions of one launch at N = 2^20 (ncu, profiles/burgers_halfstep.md)
-# over the launch's cells, e.g. P = 3: (24167170 + 41019267 + 2 x 60018446) / 2^20.
-BURGERS_FP64_FLOPS = {1: 67.17, 2: 127.37, 3: 176.64, 4: 252.11}
+# over the launch's cells, e.g. P = 3: (1048577 + 2 x 80082825) / 2^20; every
+# operation is a DFMA, so the figures are the pipe's occupancy.
+BURGERS_FP64_FLOPS = {1: 83.17, 2: 101.43, 3: 153.75, 4: 242.32}
 BURGERS_CFL = {1: 0.4, 2: 0.3, 3: 0.25, 4: 0.2}
 
 
