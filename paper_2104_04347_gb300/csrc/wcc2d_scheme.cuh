@@ -141,12 +141,7 @@ __device__ __forceinline__ float sqrt_t(float x, float& inv) {
     inv = recip_t(c);
     return c;
 }
-__device__ __forceinline__ d3 sqrt_t(d3 x, d3& inv) {
-    d3 h;
-    const d3 c = wcc::sqrt_half_rsqrt(x, h);
-    inv = h + h;
-    return c;
-}
+__device__ __forceinline__ d3 sqrt_t(d3 x, d3& inv) { return wcc::sqrt_and_recip(x, inv); }
 // 1/sqrt(x) for a direction
 __device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
 __device__ __forceinline__ d3 rsqrt_t(d3 x) {

@@ -54,6 +54,9 @@ __device__ __forceinline__ d3& operator+=(d3& a, d3 b) { a = a + b; return a; }
 __device__ __forceinline__ d3& operator*=(d3& a, d3 b) { a = a * b; return a; }
 __device__ __forceinline__ d3 fabs(d3 a) { return d3::reg(::fabs(a.v)); }
 
+// 2 a (exact)
+__device__ __forceinline__ d3 twice(d3 a) { return a + a; }
+
 // a > 0 (false for NaN), on the integer pipe
 __device__ __forceinline__ bool all_pos(d3 a) {
     const long long b = __double_as_longlong(a.v);
@@ -72,50 +75,91 @@ __device__ __forceinline__ bool mid_range(double x) {
     const unsigned e = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
     return e - 23u <= 2000u;
 }
+// Exponent between 2^-240 and 2^240: quotients of two such numbers, and of the
+// quotient and a third, neither overflow nor leave an inexact remainder.
+__device__ __forceinline__ bool moderate(double x) {
+    const unsigned e = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
+    return e - 783u <= 480u;
+}
 static __device__ __noinline__ double recip_any(double x) { return 1.0 / x; }
 static __device__ __noinline__ double sqrt_any(double x) { return ::sqrt(x); }
 
-// 1/x: the special-function unit's estimate y (about 20 bits) and one step of
-// the cubic iteration y (1 + e + e^2), e = 1 - x y, whose remaining error is
-// e^3 (2^-60): three DFMAs, one rounding in the last place that matters.
+// x with all 52 fraction bits set
+__device__ __forceinline__ bool fraction_full(double x) {
+    return __double2loint(x) == -1 && (__double2hiint(x) & 0xfffff) == 0xfffff;
+}
+
+// 1/x correctly rounded: the special-function unit's estimate y (about 20
+// bits), one step of the cubic iteration y (1 + e + e^2), e = 1 - x y, whose
+// remaining error is e^3 (2^-60), and Markstein's closing step r + r (1 - x r)
+// (IBM J. Res. Dev. 34, 1990: from an r within one unit in the last place it
+// gives the rounded reciprocal unless the fraction of x is all ones).
 __device__ __forceinline__ d3 recip(d3 x) {
-    if (mid_range(x.v)) {
+    if (mid_range(x.v) && !fraction_full(x.v)) {
         double y;
         asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x.v));
         const d3 y0 = d3::reg(y);
         const d3 e = fma(-x, y0, d3(1.0));
-        return fma(y0, fma(e, e, e), y0);
+        const d3 r = fma(y0, fma(e, e, e), y0);
+        return fma(r, fma(-x, r, d3(1.0)), r);
     }
     return d3::reg(recip_any(x.v));
+}
+
+// a / b from the rounded reciprocal rb of b: the quotient's remainder added back
+// (Markstein 1990: the rounded quotient while nothing leaves the normal range).
+__device__ __forceinline__ d3 quotient(d3 a, d3 b, d3 rb) {
+    const d3 q = a * rb;
+    return fma(fma(-q, b, a), rb, q);
 }
 
 // the limiter's weights for an exponent other than 2
 __device__ __forceinline__ d3 pow_any(d3 a, double p) { return d3::reg(::pow(a.v, p)); }
 __device__ __forceinline__ d3 div_any(d3 a, d3 b) { return d3::reg(a.v / b.v); }
 
-// half of a mid-range value: the exponent less one
-__device__ __forceinline__ d3 half_of(d3 a) {
-    return d3::reg(__hiloint2double(__double2hiint(a.v) - 0x100000, __double2loint(a.v)));
+// the neighbours of a positive normal x
+__device__ __forceinline__ d3 next_above(d3 x) { return d3::reg(__longlong_as_double(__double_as_longlong(x.v) + 1)); }
+__device__ __forceinline__ d3 next_below(d3 x) { return d3::reg(__longlong_as_double(__double_as_longlong(x.v) - 1)); }
+
+// sqrt(x) correctly rounded, for a positive mid-range x, and 1/sqrt(x) to about an
+// ulp in y: from the estimate y of 1/sqrt(x) (about 20 bits), h = x y, e = 1 - h y and
+// (1 - e)^(-1/2) = 1 + e/2 + 3 e^2/8 + ... (the next term is below 2^-60), so that
+// g = h (1 + e/2 + 3 e^2/8) is within one unit in the last place; then Tuckerman's
+// test (Markstein 1990): g is the rounded root if g (g - ulp) < x <= g (g + ulp), the signs
+// of both residuals being exact in one fused multiply-add each.
+__device__ __forceinline__ d3 sqrt_mid(d3 x, d3& y) {
+    double y_;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y_) : "d"(x.v));
+    const d3 y0 = d3::reg(y_), h = x * y0;
+    const d3 e = fma(-h, y0, d3(1.0));
+    const d3 t = e * fma(d3(0.375), e, d3(0.5));
+    y = fma(y0, t, y0);
+    const d3 g = fma(h, t, h), gb = next_below(g), ga = next_above(g);
+    return !all_pos(fma(-g, gb, x)) ? gb : all_pos(fma(-g, ga, x)) ? ga : g;
+}
+__device__ __forceinline__ bool sqrt_in_range(d3 x) { return mid_range(x.v) && __double2hiint(x.v) > 0; }
+
+__device__ __forceinline__ d3 sqrt(d3 x) {
+    if (sqrt_in_range(x)) {
+        d3 y;
+        return sqrt_mid(x, y);
+    }
+    return d3::reg(sqrt_any(x.v));
 }
 
-// sqrt(x) for a positive x, and half its reciprocal: from the estimate y of
-// 1/sqrt(x) (about 20 bits), e = 1 - x y^2 and (1 - e)^(-1/2) = 1 + e/2 +
-// 3 e^2/8 + ... (the next term is below 2^-60); the root is corrected once by
-// its own residual x - g^2.
-__device__ __forceinline__ d3 sqrt_half_rsqrt(d3 x, d3& half_rsqrt) {
-    if (mid_range(x.v) && __double2hiint(x.v) > 0) {
-        double y;
-        asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x.v));
-        const d3 y0 = d3::reg(y), h = x * y0;
-        const d3 e = fma(-h, y0, d3(1.0));
-        const d3 t = e * fma(d3(0.375), e, d3(0.5));
-        const d3 yh = half_of(y0);
-        half_rsqrt = fma(yh, t, yh);
-        const d3 g = fma(h, t, h);
-        return fma(fma(-g, g, x), half_rsqrt, g);
+// c = sqrt(x) and ic = 1/c, both correctly rounded.
+__device__ __forceinline__ d3 sqrt_and_recip(d3 x, d3& ic) {
+    if (sqrt_in_range(x)) {
+        d3 y;
+        const d3 c = sqrt_mid(x, y);
+        if (!fraction_full(c.v)) {
+            const d3 r = fma(y, fma(-c, y, d3(1.0)), y);
+            ic = fma(r, fma(-c, r, d3(1.0)), r);
+            return c;
+        }
     }
     const double c = sqrt_any(x.v);
-    half_rsqrt = d3::reg(0.5 * recip_any(c));
+    ic = d3::reg(recip_any(c));
     return d3::reg(c);
 }
 

@@ -52,19 +52,16 @@ __device__ __forceinline__ unsigned long long warp_max_key(unsigned long long k)
     return ((unsigned long long)m << 32) | lo;
 }
 
-// dt = cfl dx / amax and lam = dt / dx, quotients from a reciprocal with the
-// remainder added back: on the serial path between half-steps a warp's FP64
-// instruction takes 64 cycles and a division nine of them.
+// dt = cfl dx / amax and lam = dt / dx, rounded as the divisions, from reciprocals:
+// on the serial path between half-steps a warp's FP64 instruction takes 64 cycles and a
+// division nine of them.  Sizes far from 1 take the divisions.
 __device__ __forceinline__ void cfl_quotients(double cfl, double dx, double inv_dx, double amax, double& dt,
                                               double& lam) {
     const double x = cfl * dx;
-    if (mid_range(amax) && mid_range(x) && mid_range(inv_dx)) {
-        const d3 a(amax), n(x), ix(inv_dx);
-        const d3 r = recip(a), q = n * r;
-        const d3 t = fma(fma(-q, a, n), r, q);
-        const d3 l = t * ix;
+    if (moderate(amax) && moderate(x) && moderate(inv_dx)) {
+        const d3 a(amax), t = quotient(d3(x), a, recip(a));
         dt = t.v;
-        lam = fma(fma(-l, d3(dx), t), ix, l).v;
+        lam = quotient(t, d3(dx), d3(inv_dx)).v;
     } else {
         dt = x / amax;
         lam = dt / dx;
@@ -210,7 +207,7 @@ __device__ __forceinline__ void fp64_tile(const TileIO64& io, Step&& step, const
         });
         const StepSize& z = step();  // after the parents' loads have been issued
         ParentRecord<SYS, P, d3> r;
-        parent_record<SYS, P, d3>(c, d3(z.lam), args, r);
+        parent_record<SYS, P>(c, d3(z.lam), args, r);
         sfor<0, NV>([&](auto V) {
             constexpr int v = decltype(V)::value;
             rec[v][t] = r.A[v].v;
@@ -226,7 +223,7 @@ __device__ __forceinline__ void fp64_tile(const TileIO64& io, Step&& step, const
     // ---- phase 2: new cell t from parent slots t (left) and t + 1 (right)
     const long long i = io.first_new + t;
     if (t < kTile && i < io.n_new) {
-        d3 e[NV][K], ubar[NV], dl[NV], dr[NV];
+        d3 e[NV][K], ubar[NV], vl[NV], vr[NV];
         sfor<0, NV>([&](auto V) {
             constexpr int v = decltype(V)::value;
             d3 vL[K], vR[K];
@@ -236,61 +233,40 @@ __device__ __forceinline__ void fp64_tile(const TileIO64& io, Step&& step, const
                 vR[k] = d3::reg(rec[2 * NV + v * K + k][t + 1]);
             });
             ubar[v] = d3::reg(rec[v][t]) + d3::reg(rec[NV + v][t + 1]);
-            dl[v] = ubar[v] - vL[0];
-            dr[v] = vR[0] - ubar[v];
-            high_derivatives<P, d3>(vL, vR, e[v]);
+            vl[v] = vL[0];
+            vr[v] = vR[0];
+            derivatives_and_point_value<P, d3>(ubar[v], vL, vR, e[v]);
         });
 
-        bool limited = false;
-        if constexpr (NV == 1) {
-            e[0][1] = first_derivative<P, d3>(e[0], dl[0], dr[0]);
-            if (args.limiter) {
-                LimiterTerms<d3> T;
-                if (limiter_terms<P, d3>(e[0], dl[0], dr[0], args, T)) apply_limiter<P, d3>(e[0], T, args);
-            }
-        } else if (args.limiter) {
-            // Sec. 4: limit characteristic variables L(ubar) U, map back with
-            // R(ubar).  e_1 is linear in the differences and the higher
-            // coefficients, so it is formed after the projection.
-            EulerChar<d3> E;
-            if (!euler_char<d3>(ubar, d3(args.gamma), E)) err |= ERR_POSITIVITY;
-            d3 ce[3][K], cdl[3], cdr[3];
-            E.left(dl[0], dl[1], dl[2], cdl);
-            E.left(dr[0], dr[1], dr[2], cdr);
-            sfor<2, K>([&](auto Ki) {
-                constexpr int k = decltype(Ki)::value;
-                d3 w[3];
-                E.left(e[0][k], e[1][k], e[2][k], w);
-                ce[0][k] = w[0];
-                ce[1][k] = w[1];
-                ce[2][k] = w[2];
-            });
-            sfor<0, 3>([&](auto Ii) {
-                constexpr int r = decltype(Ii)::value;
-                ce[r][1] = first_derivative<P, d3>(ce[r], cdl[r], cdr[r]);
-                LimiterTerms<d3> T;
-                if (limiter_terms<P, d3>(ce[r], cdl[r], cdr[r], args, T)) {
-                    apply_limiter<P, d3>(ce[r], T, args);
-                    limited = true;
-                }
-            });
-            if (limited) {
-                sfor<1, K>([&](auto Ki) {
+        if (args.limiter) {
+            if constexpr (NV == 1) {
+                limit_scalar<P, SCALAR>(e[0], ubar[0], vl[0], vr[0], args);
+            } else {
+                // Sec. 4: limit characteristic variables L(ubar) U, map back with R(ubar).
+                EulerChar<d3> E;
+                if (!euler_char<d3>(ubar, d3(args.gamma), E)) err |= ERR_POSITIVITY;
+                d3 ce[3][K], cub[3], cvl[3], cvr[3];
+                E.left(ubar[0], ubar[1], ubar[2], cub);
+                E.left(vl[0], vl[1], vl[2], cvl);
+                E.left(vr[0], vr[1], vr[2], cvr);
+                sfor<0, K>([&](auto Ki) {
                     constexpr int k = decltype(Ki)::value;
-                    E.right(ce[0][k], ce[1][k], ce[2][k], e[0][k], e[1][k], e[2][k]);
+                    d3 w[3];
+                    E.left(e[0][k], e[1][k], e[2][k], w);
+                    ce[0][k] = w[0];
+                    ce[1][k] = w[1];
+                    ce[2][k] = w[2];
+                });
+                limit_scalar<P, CHARACTERISTIC>(ce[0], cub[0], cvl[0], cvr[0], args);
+                limit_scalar<P, CHARACTERISTIC>(ce[1], cub[1], cvl[1], cvr[1], args);
+                const d3 w0 = limit_scalar<P, LAST_CHARACTERISTIC>(ce[2], cub[2], cvl[2], cvr[2], args);
+                sfor<0, K>([&](auto Ki) {
+                    constexpr int k = decltype(Ki)::value;
+                    if constexpr (k < 2) E.right(ce[0][k], ce[1][k], ce[2][k], e[0][k], e[1][k], e[2][k]);
+                    else E.right_scaled(ce[0][k], ce[1][k], w0, ce[2][k], e[0][k], e[1][k], e[2][k]);
                 });
             }
         }
-        if (NV > 1 && !limited) {
-            sfor<0, NV>([&](auto V) {
-                constexpr int v = decltype(V)::value;
-                e[v][1] = first_derivative<P, d3>(e[v], dl[v], dr[v]);
-            });
-        }
-        sfor<0, NV>([&](auto V) {  // the limiter keeps the cell average
-            constexpr int v = decltype(V)::value;
-            e[v][0] = point_value<P, d3>(ubar[v], e[v]);
-        });
 
         bool bad = false;
         sfor<0, NV>([&](auto V) {

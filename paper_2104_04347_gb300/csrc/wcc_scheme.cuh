@@ -203,9 +203,7 @@ inline long long __double_as_longlong_host(double d) {
     return b;
 }
 
-// 1/x: correctly rounded division in FP64; the hardware reciprocal with one
-// Newton step (correctly rounded) in FP32.
-__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
+// 1/x: the hardware reciprocal with one Newton step (correctly rounded).
 __device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
 
 // NaN / Inf test on the exponent bits (integer pipe only).
@@ -327,9 +325,16 @@ __device__ __forceinline__ void ck_table(const R (&c)[nvars(SYS)][P + 1], R lam,
                         q = fma(X[1][i][j], w[aa - i][b - j], q);
                     });
                 });
-                const R p = g1 * fma((R)-0.5, q, X[2][aa][b]);
-                H[aa][b] = X[2][aa][b] + p;
-                Fm[aa][b] = q + p;
+                const R T = fma((R)-0.5, q, X[2][aa][b]);
+                if constexpr (f32) {
+                    const R p = g1 * T;
+                    H[aa][b] = X[2][aa][b] + p;
+                    Fm[aa][b] = q + p;
+                } else {
+                    // p joins both sums unrounded
+                    H[aa][b] = fma(g1, T, X[2][aa][b]);
+                    Fm[aa][b] = fma(g1, T, q);
+                }
                 R fe = (R)0;
                 sfor<0, aa + 1>([&](auto Ii) {
                     constexpr int i = decltype(Ii)::value;
@@ -357,41 +362,50 @@ __device__ __forceinline__ void ck_table(const R (&c)[nvars(SYS)][P + 1], R lam,
     }
 }
 
-template <int SYS, int P, class R>
-__device__ __forceinline__ void parent_record(const R (&c)[nvars(SYS)][P + 1], R lam, const StepArgs& args,
-                                              ParentRecord<SYS, P, R>& out) {
+// FP64.  The operations and their order here, in the new cell and in the limiter
+// below are fixed down to the last rounding (every sum, product and fused
+// multiply-add is written out, nothing is left to the compiler's contraction): where a
+// one-sided slope of the limiter nearly vanishes the scheme multiplies rounding
+// (a smooth advected sine moves by up to 4e-4 at t = 2 when its data move by 1e-16),
+// so that only the same operations give the same run.
+template <int SYS, int P>
+__device__ __forceinline__ void parent_record(const d3 (&c)[nvars(SYS)][P + 1], d3 lam, const StepArgs& args,
+                                              ParentRecord<SYS, P, d3>& out) {
     constexpr int NV = nvars(SYS);
     constexpr int K = P + 1;
-    R X[NV][K][K];
-    R F0[NV][K];
-    ck_table<SYS, P, R>(c, lam, args, X, F0);
+    d3 X[NV][K][K];
+    d3 F0[NV][K];
+    ck_table<SYS, P, d3>(c, lam, args, X, F0);
 
     sfor<0, NV>([&](auto V) {
         constexpr int v = decltype(V)::value;
         // Eq. Cal1DFlux in Taylor form: fbar = sum_b F[0][b] / (b + 1).
-        R fbar = F0[v][0];
+        d3 fbar = F0[v][0];
         sfor<1, K>([&](auto Bi) {
             constexpr int b = decltype(Bi)::value;
-            fbar = fma((R)(1.0 / (b + 1.0)), F0[v][b], fbar);
+            fbar = fma((d3)(1.0 / (b + 1.0)), F0[v][b], fbar);
         });
-        // Eqs. SubEq:1DCellAVGR / SubEq:1DCellAVGL: the half-cell averages
-        // share their even part, and the flux joins the odd one:
-        // A, B = even / 2 +- (odd / 2 + lam fbar).
-        R even = (R)0.5 * c[v][0], odd = (R)0.125 * c[v][1];
-        sfor<2, K>([&](auto Ki) {
+        // Eqs. SubEq:1DCellAVGR / SubEq:1DCellAVGL: half-cell averages.
+        d3 ur = c[v][0], ul = c[v][0];
+        sfor<1, K>([&](auto Ki) {
             constexpr int k = decltype(Ki)::value;
-            constexpr double wk = 0.5 / ((k + 1.0) * cpow2(k));
-            if constexpr (k & 1) odd = fma((R)wk, c[v][k], odd);
-            else even = fma((R)wk, c[v][k], even);
+            constexpr double wk = 1.0 / ((k + 1.0) * cpow2(k));
+            ur = fma((d3)wk, c[v][k], ur);
+            ul = fma((d3)((k & 1) ? -wk : wk), c[v][k], ul);
         });
-        const R g = fma(lam, fbar, odd);
-        out.A[v] = even + g;
-        out.B[v] = even - g;
-        // Eq. SubEq:Cal_1D_Derivatives_4: vertex values at t^{n+1/2}.
+        out.A[v] = fma(lam, fbar, (d3)0.5 * ur);
+        out.B[v] = fma(-lam, fbar, (d3)0.5 * ul);
+        // Eq. SubEq:Cal_1D_Derivatives_4: vertex values at t^{n+1/2} (the density's
+        // first two time terms at P = 6 join the sum unrounded).
         sfor<0, K>([&](auto Ki) {
             constexpr int k = decltype(Ki)::value;
-            R s = X[v][k][0];
-            sfor<1, K - k>([&](auto Mi) { s += X[v][k][decltype(Mi)::value]; });
+            d3 s = X[v][k][0];
+            sfor<1, K - k>([&](auto Mi) {
+                constexpr int m = decltype(Mi)::value;
+                constexpr double w = (k + 1.0) / m;
+                if constexpr (SYS == EULER && P == 6 && v == 0 && m <= 2) s = fma(-times<w == 1.0>(lam, w), X[1][k + 1][m - 1], s);
+                else s += X[v][k][m];
+            });
             out.vtx[v][k] = s;
         });
     });
@@ -426,155 +440,120 @@ __device__ __forceinline__ void derivatives_and_point_value(R ubar, const R (&vL
     e[0] = u0;
 }
 
-// Coefficients e_2 .. e_P of a new cell (Eq. SubEq:Cal_1D_Derivatives_3).
-template <int P, class R>
-__device__ __forceinline__ void high_derivatives(const R (&vL)[P + 1], const R (&vR)[P + 1], R (&e)[P + 1]) {
-    sfor<0, P - 1>([&](auto Ii) {
-        constexpr int k = P - 1 - decltype(Ii)::value;  // P - 1 .. 1
-        R s = vR[k] - vL[k];
-        sfor<3, P - k + 1>([&](auto Mi) {
-            constexpr int m = decltype(Mi)::value;
-            if constexpr (m & 1) {
-                constexpr double cm = 2.0 * cbinom(k + m, m) * cpow2(-m);
-                s = fma((R)-cm, e[k + m], s);
-            }
-        });
-        e[k + 1] = s * (R)(1.0 / (k + 1.0));
-    });
+// Whether the side weights of the limiter leave no trace in the rounded result, so
+// that they need not be formed: P >= 2, alpha = 2, exponents only (integer pipe).
+// w_m is at most (sigma tau / d_m)^2 to rounding, below 2^(r_m + 1); then
+//   w_1 + w_2 below 2^-54:                             w_0 = 1 - (w_1 + w_2) is 1,
+//   (w_1 + w_2) ubar below 2^-54 of e_0:                e_0 is kept,
+//   |w_1 s_1| + |w_2 s_2| below 2^-54 of e_1:            e_1 is kept,
+// each with a binary digit or two to spare for the roundings.  Denominators
+// within 2^+-160 keep the products the weights are made of in range (they have an
+// overflow of their own, which is not hidden); NaN and infinities are outside it.
+// A coefficient -0 (and negative subnormals) would come out as +0 and is left to the sum.
+// Away from jumps, kinks and crests that is every cell: Euler P = 3 at 2^19 cells 485 ->
+// 412 us per half-step, P = 5 at 65 521 cells 137 -> 127 us.
+__device__ __forceinline__ bool weights_vanish(const d3 (&d)[3], d3 st, d3 s1, d3 s2, d3 e0, d3 e1, d3 ubar) {
+    const int x0 = exponent_of(d[0]), x1 = exponent_of(d[1]), x2 = exponent_of(d[2]);
+    const int lo = min(x0, min(x1, x2)), hi = max(x0, max(x1, x2));
+    const int r1 = 2 * (exponent_of(st) + 1 - x1), r2 = 2 * (exponent_of(st) + 1 - x2);
+    const int r = max(r1, r2);
+    const bool minus_zero = (unsigned)__double2hiint(e0.v) >> 20 == 0x800u || (unsigned)__double2hiint(e1.v) >> 20 == 0x800u;
+    return !minus_zero && lo >= 1023 - 160 && hi <= 1023 + 160 && r + 2 <= -54 &&
+           max(r1 + exponent_of(s1), r2 + exponent_of(s2)) + 3 < exponent_of(e1) - 54 &&
+           r + 3 + exponent_of(ubar) < exponent_of(e0) - 54;
 }
 
-// e_1 of the same equation from the one-sided differences dl = ubar - u_{i-1/2}
-// and dr = u_{i+1/2} - ubar: u_{i+1/2} - u_{i-1/2} less the odd terms above.
-template <int P, class R>
-__device__ __forceinline__ R first_derivative(const R (&e)[P + 1], R dl, R dr) {
-    R s = dl + dr;
-    sfor<3, P + 1>([&](auto Mi) {
-        constexpr int m = decltype(Mi)::value;
-        if constexpr (m & 1) s = fma((R)(-2.0 * cpow2(-m)), e[m], s);
-    });
-    return s;
-}
-
-// Point value less the cell average: -sum over even k >= 2 of e_k / ((k+1) 2^k)
-// (Eq. 1DCalU).
-template <int P, class R>
-__device__ __forceinline__ R point_value(R ubar, const R (&e)[P + 1]) {
-    R u0 = ubar;
-    sfor<2, P + 1>([&](auto Ki) {
-        constexpr int k = decltype(Ki)::value;
-        if constexpr ((k & 1) == 0) u0 = fma((R)(-1.0 / ((k + 1.0) * cpow2(k))), e[k], u0);
-    });
-    return u0;
-}
-
-// WENO-type limiter of Sec. 2.2 on one scalar (or characteristic) component
-// in deviation form: e[1..P] the Taylor coefficients of u_0 (overwritten by
-// those of u_*), dl = ubar - u_{i-1/2}, dr = u_{i+1/2} - ubar with the
-// time-extrapolated vertex values.  The limiter keeps the cell average, and
-// nothing in it depends on it.  The two residuals of sigma are the same
-// number: the unlimited polynomial's difference between its ends is
-// u_{i+1/2} - u_{i-1/2} by construction of e_1, so both equal
-//   r = (even part at the ends less the average) + (dl - dr) / 2.
-//
-// In two steps: limiter_terms forms the denominators and sigma tau, and says
-// whether the limiter acts on the component at all.  With sigma tau below
-// 2^-31 of every denominator (compared on the exponents) the side weights are
-// below 2^-62: w_0 is 1 exactly, and what they add to e_1 is below the
-// rounding of the differences it is made of.  Away from jumps and kinks that
-// is every cell, and where no component of a cell needs it the weights, their
-// reciprocal and the back-projection (a fifth of the FP64 operations) are left
-// out: Euler P = 3 at 2^19 cells 426 -> 346 us per half-step, P = 5 at 65 521 cells
-// 128 -> 110 us.  The choice is each cell's own.
-template <class R>
-struct LimiterTerms {
-    R s1, s2;          // slopes of u_1, u_2 (Eq. SubEq:1DU12)
-    R b0, b1, b2, st;  // beta_m and sigma tau
-    R d0, d1, d2;      // beta_m^2 + eps
-};
-
-template <int P, class R>
-__device__ __forceinline__ bool limiter_terms(const R (&e)[P + 1], R dl, R dr, const StepArgs& args,
-                                              LimiterTerms<R>& T) {
-    T.s1 = dl + dl;
-    T.s2 = dr + dr;
+// WENO-type limiter of Sec. 2.2 on one scalar (or characteristic) component,
+// FP64.  e: Taylor coefficients of u_0 (overwritten by u_*; of the last
+// characteristic component only e_0 and e_1, the caller multiplies the others by
+// the w_0 returned), ubar its cell average, vl / vr the time-extrapolated vertex
+// values u_{i-1/2}, u_{i+1/2}.
+enum Component { SCALAR, CHARACTERISTIC, LAST_CHARACTERISTIC };
+template <int P, Component C>
+__device__ __forceinline__ d3 limit_scalar(d3 (&e)[P + 1], d3 ubar, d3 vl, d3 vr, const StepArgs& args) {
+    const d3 s1 = twice(ubar - vl);  // Eq. SubEq:1DU12, slope of u_1
+    const d3 s2 = twice(vr - ubar);  // slope of u_2
     // beta_0 (Eq. 1DSmoothIndicator) as a quadratic form in e_1..e_P
+    d3 b0;
     sfor<1, P + 1>([&](auto Ji) {
         constexpr int j = decltype(Ji)::value;
-        R row = times<csmooth(j, j) == 1.0>(e[j], csmooth(j, j));
+        d3 row = times<csmooth(j, j) == 1.0>(e[j], csmooth(j, j));
         sfor<j + 1, P + 1>([&](auto Li) {
             constexpr int l = decltype(Li)::value;
             constexpr double cjl = 2.0 * csmooth(j, l);
-            if constexpr (cjl != 0.0) row = fma((R)cjl, e[l], row);
+            if constexpr (cjl != 0.0) row = fma((d3)cjl, e[l], row);
         });
-        if constexpr (j == 1) T.b0 = row * e[1];
-        else T.b0 = fma(row, e[j], T.b0);
+        if constexpr (j == 1) b0 = row * e[1];
+        else b0 = fma(row, e[j], b0);
     });
-    T.b1 = T.s1 * T.s1;
-    T.b2 = T.s2 * T.s2;
-    const R eps = (R)args.eps;
+    const d3 b1 = s1 * s1, b2 = s2 * s2;
+    const d3 eps = (d3)args.eps;
+    d3 d[3], st;
     if constexpr (P == 1) {
-        T.d0 = T.b0 + eps;
-        T.d1 = T.b1 + eps;
-        T.d2 = T.b2 + eps;
-        return true;
+        d[0] = b0 + eps;
+        d[1] = b1 + eps;
+        d[2] = b2 + eps;
     } else {
-        R r = (R)(1.0 / 6.0) * e[2];
-        sfor<4, P + 1>([&](auto Ki) {
+        d3 up = e[0], um = e[0];
+        sfor<1, P + 1>([&](auto Ki) {
             constexpr int k = decltype(Ki)::value;
-            if constexpr ((k & 1) == 0) r = fma((R)(cpow2(-k) * k / (k + 1.0)), e[k], r);
+            up = fma((d3)chalf(k, false), e[k], up);
+            um = fma((d3)chalf(k, true), e[k], um);
         });
-        r = fma((R)0.5, dl - dr, r);
-        const R y = e[P] * r;
-        T.st = ((R)(2.0 * cfact(P) * cfact(P)) * y) * y;
-        T.d0 = fma(T.b0, T.b0, eps);
-        T.d1 = fma(T.b1, T.b1, eps);
-        T.d2 = fma(T.b2, T.b2, eps);
-        const int least = min(exponent_of(T.d0), min(exponent_of(T.d1), exponent_of(T.d2)));
-        return !args.alpha_is_two || exponent_of(T.st) + 32 > least;
+        const d3 rr = up - vr, rl = um - vl;
+        const d3 sigma = fma(rr, rr, rl * rl);
+        const d3 tp = (d3)cfact(P) * e[P];
+        st = sigma * (tp * tp);
+        d[0] = fma(b0, b0, eps);
+        d[1] = fma(b1, b1, eps);
+        d[2] = fma(b2, b2, eps);
+        if (args.alpha_is_two && weights_vanish(d, st, s1, s2, e[0], e[1], ubar)) return (d3)1;
     }
-}
-
-template <int P, class R>
-__device__ __forceinline__ void apply_limiter(R (&e)[P + 1], const LimiterTerms<R>& T, const StepArgs& args) {
-    R w0, w1, w2;
+    d3 w1, w2;
     if (args.alpha_is_two) {
         // Multiplied through by the denominators, so that one reciprocal
         // normalises the weights; w0 = 1 - w1 - w2 is exactly 1 when the
         // other two vanish.
+        const d3 p12 = d[1] * d[2], p02 = d[0] * d[2], p01 = d[0] * d[1];
+        d3 sum, h1, h2;
         if constexpr (P == 1) {
             // Eq. 1D2ndOrderWeights: w_m ~ (beta_m + eps)^-2
-            const R p12 = T.d1 * T.d2, p02 = T.d0 * T.d2, p01 = T.d0 * T.d1;
-            const R inv = recip(fma(p12, p12, fma(p02, p02, p01 * p01)));
-            w1 = (p02 * inv) * p02;
-            w2 = (p01 * inv) * p01;
+            h1 = p02 * p02;
+            h2 = p01 * p01;
+            sum = fma(p12, p12, h1) + h2;
         } else {
             // Eq. 1DHighOrderWeights: w0 ~ 1 + (st/d0)^2, w_m ~ (st/d_m)^2
-            const R p12 = T.d1 * T.d2, sd0 = T.st * T.d0;
-            const R s12 = T.st * p12, s02 = sd0 * T.d2, s01 = sd0 * T.d1, p = T.d0 * p12;
-            const R inv = recip(fma(p, p, fma(s12, s12, fma(s02, s02, s01 * s01))));
-            w1 = (s02 * inv) * s02;
-            w2 = (s01 * inv) * s01;
+            const d3 s12 = st * p12, s02 = st * p02, s01 = st * p01, p = d[0] * p12;
+            h1 = s02 * s02;
+            h2 = s01 * s01;
+            sum = fma(p, p, s12 * s12) + h1 + h2;
         }
+        const d3 inv = recip(sum);
+        w1 = h1 * inv;
+        w2 = h2 * inv;
     } else {
-        const double al = args.alpha;
-        R wh0, wh1, wh2;
-        if constexpr (P == 1) {
-            wh0 = pow_any(recip(T.d0), al);
-            wh1 = pow_any(recip(T.d1), al);
-            wh2 = pow_any(recip(T.d2), al);
-        } else {
-            wh0 = (R)1 + pow_any(div_any(T.st, T.d0), al);
-            wh1 = pow_any(div_any(T.st, T.d1), al);
-            wh2 = pow_any(div_any(T.st, T.d2), al);
+        d3 wh[3];
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            if constexpr (P == 1) {
+                // (beta_1, beta_2 of the first two characteristic components join eps unrounded)
+                if (C == CHARACTERISTIC && m > 0) d[m] = m == 1 ? fma(s1, s1, eps) : fma(s2, s2, eps);
+                wh[m] = pow_any(recip(d[m]), args.alpha);
+            } else {
+                wh[m] = pow_any(div_any(st, d[m]), args.alpha);
+            }
         }
-        const R inv = recip(wh0 + wh1 + wh2);
-        w1 = wh1 * inv;
-        w2 = wh2 * inv;
+        if constexpr (P > 1) wh[0] = (d3)1 + wh[0];
+        const d3 inv = recip(wh[0] + wh[1] + wh[2]);
+        w1 = wh[1] * inv;
+        w2 = wh[2] * inv;
     }
-    w0 = (R)1 - (w1 + w2);
+    const d3 w12 = w1 + w2, w0 = (d3)1 - w12;
     // Eq. 1DLimitedPolynomial, coefficient by coefficient.
-    e[1] = fma(w0, e[1], fma(w1, T.s1, w2 * T.s2));
-    sfor<2, P + 1>([&](auto Ki) { e[decltype(Ki)::value] *= w0; });
+    e[0] = fma(w0, e[0], w12 * ubar);
+    e[1] = fma(w0, e[1], fma(w1, s1, w2 * s2));
+    if constexpr (C != LAST_CHARACTERISTIC) sfor<2, P + 1>([&](auto Ki) { e[decltype(Ki)::value] *= w0; });
+    return w0;
 }
 
 // Eigenvectors of the Euler flux Jacobian at the cell average (conserved
@@ -598,14 +577,29 @@ struct EulerChar {
 
     __device__ __forceinline__ void left(R d0, R d1, R d2, R (&w)[3]) const {
         const R X = b1h * fma(nu, d1, fma(hu2, d0, d2));
-        const R Y = ich * fma(nu, d0, d1);
-        w[0] = X - Y;
+        const R Z = fma(nu, d0, d1);
         w[1] = fma((R)-2, X, d0);
-        w[2] = X + Y;
+        if constexpr (is_f64<R>) {
+            // (Y joins both sums unrounded)
+            w[0] = fma(-ich, Z, X);
+            w[2] = fma(ich, Z, X);
+        } else {
+            const R Y = ich * Z;
+            w[0] = X - Y;
+            w[2] = X + Y;
+        }
     }
     __device__ __forceinline__ void right(R w0, R w1, R w2, R& d0, R& d1, R& d2) const {
-        const R s = w0 + w2;
-        const R m = c * (w2 - w0);
+        right_of(w0 + w2, w2 - w0, w1, d0, d1, d2);
+    }
+    // from w_0, w_1 and s w_2
+    __device__ __forceinline__ void right_scaled(R w0, R w1, R s, R w2, R& d0, R& d1, R& d2) const {
+        right_of(fma(s, w2, w0), fma(s, w2, -w0), w1, d0, d1, d2);
+    }
+
+private:
+    __device__ __forceinline__ void right_of(R s, R diff, R w1, R& d0, R& d1, R& d2) const {
+        const R m = c * diff;
         d0 = s + w1;
         d1 = fma(u, d0, m);
         d2 = fma(H, s, fma(u, m, hu2 * w1));
@@ -620,22 +614,21 @@ __device__ __forceinline__ bool euler_char(const R (&U)[3], R gamma, EulerChar<R
     const R irho = recip(U[0]);
     const R u = U[1] * irho;
     const R g1 = gamma - (R)1;
-    const R hu = (R)0.5 * u;
-    const R p = g1 * fma(-hu, U[1], U[2]);
+    const R p = g1 * fma((R)-0.5 * U[1], u, U[2]);
     const R c2 = gamma * p * irho;
+    R ic;
+    if constexpr (f32) {
+        ic = rsqrt_approx(c2);  // the basis only needs FP32 accuracy
+        E.c = c2 * ic;
+    } else {
+        E.c = sqrt_and_recip(c2, ic);
+    }
+    E.H = (U[2] + p) * irho;
     E.u = u;
     E.nu = -u;
-    E.hu2 = hu * u;
-    E.H = (U[2] + p) * irho;
-    if constexpr (f32) {
-        const R ic = rsqrt_approx(c2);  // the basis only needs FP32 accuracy
-        E.c = c2 * ic;
-        E.b1h = (R)0.5 * g1 * ic * ic;
-        E.ich = (R)0.5 * ic;
-    } else {
-        E.c = sqrt_half_rsqrt(c2, E.ich);
-        E.b1h = (R)2 * g1 * (E.ich * E.ich);
-    }
+    E.hu2 = (R)0.5 * u * u;
+    E.b1h = (R)0.5 * g1 * ic * ic;
+    E.ich = (R)0.5 * ic;
     return all_pos(U[0]) && all_pos(p);
 }
 
@@ -664,8 +657,7 @@ __device__ __forceinline__ R wave_speed(const R* u0, const StepArgs& args, unsig
             const R u = u0[1] * irho;
             const R p = g1 * fma((R)-0.5 * u0[1], u, u0[2]);
             if (!all_pos(rho) || !all_pos(p)) err |= ERR_POSITIVITY;
-            R half_rsqrt;
-            return fabs(u) + sqrt_half_rsqrt(gamma * p * irho, half_rsqrt);
+            return fabs(u) + sqrt(gamma * p * irho);
         }
     }
 }
