@@ -1,7 +1,8 @@
-"""FP64 1D marches give the same bits as ever: SHA-256 digests of the stage and the
-dt list of marches recorded on a GB300 from the library as its FP64 kernels first were
-(tests/golden/fp64_marches_1d.txt), for every system, degree, boundary, limiter
-option and route (one cluster of CTAs, or single half-steps on larger meshes).
+"""1D marches give the same bits as ever: SHA-256 digests of the stage and the dt list
+of marches recorded on a GB300 from the library as its kernels first were
+(tests/golden/fp64_marches_1d.txt, mixed_marches_1d.txt), for every system, degree,
+boundary, limiter option and route (one cluster of CTAs, single half-steps on larger
+meshes, FP32-mixed also two half-steps per launch and batches).
 
 Bits, because no tolerance would do: where a one-sided slope of the limiter nearly
 vanishes, or behind a shock, the scheme multiplies rounding, and after some hundred
@@ -18,7 +19,7 @@ from paper_2104_04347_gb300 import inputs, wcc
 
 pytestmark = pytest.mark.gpu
 
-GOLDEN = os.path.join(os.path.dirname(os.path.abspath(__file__)), "golden", "fp64_marches_1d.txt")
+GOLDEN = os.path.join(os.path.dirname(os.path.abspath(__file__)), "golden")
 CFL = {1: 0.4, 2: 0.3, 3: 0.25, 4: 0.22, 5: 0.16, 6: 0.14}
 
 
@@ -97,6 +98,39 @@ def marches():
     return out
 
 
+def mixed_marches():
+    out = {}
+    B, E, PER, TR, A = inputs.BURGERS, inputs.EULER, inputs.PERIODIC, inputs.TRANSMISSIVE, inputs.ADVECTION
+    for P in range(1, 7):
+        for N in (200, 3000, 5000):
+            for tb in (1, 2):
+                o = {"precision": wcc.FP32_MIXED, "tb_depth": tb}
+                out[f"wave P{P} N{N} depth {tb}"] = (E, N, P, (0.0, 1.0), PER, lambda N=N, P=P: _wave(N, P, 0.7, PER), ("step", 60), o)
+                out[f"tube P{P} N{N} depth {tb}"] = (E, N, P, (0.0, 1.0), TR, lambda N=N, P=P: _tube(N, P), ("step", 30), o)
+            o = {"precision": wcc.FP32_MIXED}
+            out[f"burgers P{P} N{N}"] = (B, N, P, (0.0, 2.0), PER, lambda N=N, P=P: _sine(N, P, 0.25, 0.7, 0.5), ("step", 60), o)
+            out[f"advection P{P} N{N}"] = (A, N, P, (0.0, 2.0), PER, lambda N=N, P=P: _sine(N, P, 0.25, 0.7, 0.5), ("step", 60), o)
+    return out
+
+
+class _Member:
+    def __init__(self, N, P, bc, q):
+        self.system, self.N, self.P, self.x_l, self.x_r, self.bc, self.q0 = inputs.EULER, N, P, 0.0, 1.0, bc, q
+
+
+def batch_digest():
+    members = [_Member(N, P, inputs.TRANSMISSIVE, _tube(N, P)) if N % 2 else _Member(N, P, inputs.PERIODIC, _wave(N, P, 0.7, inputs.PERIODIC))
+               for N, P in ((200, 2), (301, 3), (777, 2), (1500, 3), (2601, 3))]
+    with wcc.Batch(members) as b:
+        b.set_initial([m.q0 for m in members])
+        b.step(30, CFL[3])
+        h = hashlib.sha256()
+        for i, q in enumerate(b.get_dofs()):
+            h.update((np.ascontiguousarray(q) + 0.0).tobytes())
+            h.update(np.ascontiguousarray(b.dt_history(i)).tobytes())
+    return h.hexdigest()
+
+
 def digest(march):
     system, N, P, domain, bc, data, how, options = march
     with wcc.Solver(system, N, P, domain, bc, **options) as s:
@@ -109,13 +143,20 @@ def digest(march):
     return hashlib.sha256((np.ascontiguousarray(q) + 0.0).tobytes() + np.ascontiguousarray(dts).tobytes()).hexdigest()
 
 
-def _recorded():
-    if not os.path.exists(GOLDEN):
-        return {}
-    with open(GOLDEN) as f:
+def _recorded(name):
+    with open(os.path.join(GOLDEN, name)) as f:
         return dict(line.rstrip("\n").rsplit("  ", 1) for line in f if line.strip())
 
 
 @pytest.mark.parametrize("name", list(marches()))
 def test_same_bits(name):
-    assert digest(marches()[name]) == _recorded()[name]
+    assert digest(marches()[name]) == _recorded("fp64_marches_1d.txt")[name]
+
+
+@pytest.mark.parametrize("name", list(mixed_marches()))
+def test_same_bits_mixed(name):
+    assert digest(mixed_marches()[name]) == _recorded("mixed_marches_1d.txt")[name]
+
+
+def test_same_bits_batch():
+    assert batch_digest() == _recorded("mixed_marches_1d.txt")["batch"]
