@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(kThreadsMixed) halfstep_small(const StepArgs a
         if constexpr (F32) return (double)__uint_as_float(k);
         else return __longlong_as_double((long long)k);
     };
-    Key sized_key = 0;  // the bound that z's quotients were taken from (none at first)
+    Key sized_key = ~Key(0);  // the bound that z's quotients were taken from (none at first: no speed has these bits)
     int sized = -1;  // the half-step that z belongs to
     auto step = [&]() -> const StepSize& {
         if (sized == s) return z;
