@@ -360,20 +360,21 @@ __device__ __forceinline__ bool limiter_acts_f2(const f2 (&d)[P + 1], f2 dl, f2 
 // estimates and some thirty other instructions) out where it does not: Euler
 // P = 3 at 2^22 cells 127.5 -> 122.9 us per half-step, two half-steps per launch at
 // P = 2 24.7 -> 23.0 us.
-template <int P, bool ASK = true>
-__device__ __forceinline__ void limit_deviation_f2(f2 (&d)[P + 1], f2 dl, f2 dr, const StepArgs& args) {
+template <int P, bool ASK = true, bool SCALE = true>
+__device__ __forceinline__ f2 limit_deviation_f2(f2 (&d)[P + 1], f2 dl, f2 dr, const StepArgs& args) {
     f2 b0, b1, b2, w0, w1, w2;
     const f2 st = limiter_betas_f2<P>(d, dl, dr, b0, b1, b2);
     if constexpr (P == 1) {
         weights_p1_f2(b0, b1, b2, args, w0, w1, w2);
     } else {
-        if (ASK && !limiter_acts_f2(b0, b1, b2, st, args)) return;
+        if (ASK && !limiter_acts_f2(b0, b1, b2, st, args)) return f2(1.f);
         weights_hi_f2(b0, b1, b2, st, args, w0, w1, w2);
     }
     const f2 s1 = f2(2.f) * dl, s2 = f2(2.f) * dr;
     d[0] *= w0;
     d[1] = fma(w0, d[1], fma(w1, s1, w2 * s2));
-    sfor<2, P + 1>([&](auto Ki) { d[decltype(Ki)::value] *= w0; });
+    if constexpr (SCALE) sfor<2, P + 1>([&](auto Ki) { d[decltype(Ki)::value] *= w0; });
+    return w0;
 }
 
 // ------------------------------------------------------ the paired tile
@@ -611,16 +612,18 @@ __device__ __forceinline__ void mixed_new_cells(const float2* rec, const StepArg
                     acts |= limiter_acts_f2<P>(cd[rr], cdl[rr], cdr[rr], args);
                 });
             }
+            f2 w0(1.f);  // of the last component, whose e_2 .. join the back-projection's sums unrounded
             if (acts) {
                 sfor<0, 3>([&](auto Ii) {
                     constexpr int rr = decltype(Ii)::value;
                     cd[rr][0] = -average_minus_centre<P>(cd[rr]);
-                    limit_deviation_f2<P, !SMALL>(cd[rr], cdl[rr], cdr[rr], args);
+                    w0 = limit_deviation_f2<P, !SMALL, (rr < 2)>(cd[rr], cdl[rr], cdr[rr], args);
                 });
             }
             sfor<1, K>([&](auto Ki) {
                 constexpr int k = decltype(Ki)::value;
-                E.right(cd[0][k], cd[1][k], cd[2][k], d[0][k], d[1][k], d[2][k]);
+                if constexpr (k < 2) E.right(cd[0][k], cd[1][k], cd[2][k], d[0][k], d[1][k], d[2][k]);
+                else E.right_scaled(cd[0][k], cd[1][k], w0, cd[2][k], d[0][k], d[1][k], d[2][k]);
             });
             sfor<0, 3>([&](auto Vi) {
                 constexpr int v = decltype(Vi)::value;
