@@ -85,6 +85,13 @@ enum {
  * above); plain FP32 only its default; FP64 only 127.  Other values are
  * WCC_E_INVAL.  wcc_autotune picks it, with tb_depth, by timing.
  *
+ * Small meshes: in FP64 (up to 2032 cells in a stage) and FP32-mixed at P <= 4
+ * (up to 4080) one cluster of CTAs holds the mesh and marches up to 256
+ * half-steps per launch, in wcc_step(nsteps >= 2) and wcc_step_until with
+ * tb_depth = 1.  The results are the same bit for bit.  cells_per_block other
+ * than 0 asks for the one-half-step kernel with that tile, graph_chunk = 0 for
+ * one launch per half-step; both are taken as asked on small meshes too.
+ *
  * tb_depth (temporal blocking): half-steps per pass over the state in
  * device memory, 1 or 2 (0 reads as 1).  With 2 (FP32 variants only,
  * WCC_E_INVAL with WCC_FP64 or a batch), wcc_step advances the stage two
@@ -151,8 +158,8 @@ int wcc_step(wcc_handle h, int64_t nsteps, double cfl);
 
 /* Autotuner of the single-grid launch: times every compiled launch
  * configuration of the handle -- for FP32-mixed cells_per_block 255 and 510
- * with one half-step per launch, and two half-steps per launch -- on the
- * handle's own current stage at CFL number cfl (a warm-up graph, then three
+ * with one half-step per launch, on a small mesh also the cluster (0), and two
+ * half-steps per launch -- on the handle's own current stage at CFL number cfl (a warm-up graph, then three
  * graphs of graph_chunk half-steps each, CUDA events on the handle's
  * stream), keeps the fastest in the handle's options and reports it in
  * *cells_per_block and *tb_depth (either may be NULL).  The stage, its time

@@ -428,12 +428,16 @@ cudaError_t launch_small_kernel(wcc_ctx* h, const StepArgs& a, int nsteps, doubl
     }
 }
 
-// nsteps single CFL half-steps: in clusters where one holds the mesh, else in
+// Does one cluster march the mesh?  Not where the options ask for a tile size
+// (cells_per_block) or for a launch per half-step (graph_chunk = 0).
+bool clustered(const wcc_ctx* h) { return h->small_ctas && h->opt.cells_per_block == 0 && h->opt.graph_chunk >= 2; }
+
+// nsteps single CFL half-steps: in clusters where one marches the mesh, else in
 // graphs of graph_chunk, then direct launches.
 int step_single(wcc_ctx* h, long long nsteps, double cfl) {
     int rc;
     long long left = nsteps;
-    while (h->small_ctas && left >= 2) {
+    while (clustered(h) && left >= 2) {
         const int k = (int)std::min<long long>(left, kSmallSteps);
         cudaError_t e = launch_small_kernel(h, make_args(h, h->cur, h->parity, cfl, 0.0), k, INFINITY, nullptr);
         if (e != cudaSuccess) return cuda_fail(h, e, "small-mesh launch");
@@ -752,9 +756,10 @@ int wcc_autotune(wcc_handle h, double cfl, int* cells_per_block, int* tb_depth) 
     struct Cand {
         int cpb, tb;
     };
-    Cand cands[3];
+    Cand cands[4];
     int nc = 0;
     if (h->opt.precision == WCC_FP32_MIXED) {
+        if (h->small_ctas && h->opt.graph_chunk >= 2) cands[nc++] = {0, 1};  // the cluster
         cands[nc++] = {kTileMixed, 1};
         cands[nc++] = {2 * kTileMixed, 1};
         cands[nc++] = {0, 2};
@@ -917,7 +922,7 @@ int wcc_step_until(wcc_handle h, double t_end, double cfl, int64_t* nsteps_taken
     // the rule below before every half-step (advection, 200 cells, 800 half-steps:
     // 2.8 ms; 7.0 ms in graphs with a wait for the device state after each and, for
     // the last 128 half-steps, after every half-step).
-    while (h->small_ctas && h->opt.tb_depth == 1) {
+    while (clustered(h) && h->opt.tb_depth == 1) {
         const double dt = next_dt(s);
         if (!(dt > 0.0) || !(t_end - s.t >= 2.0 * dt * (1.0 - 1e-12))) break;
         if ((rc = ensure_history(h, h->steps + kSmallSteps + 2)) != WCC_OK) return finish(rc);
