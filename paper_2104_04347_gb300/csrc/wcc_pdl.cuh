@@ -2,12 +2,20 @@
 // (programmatic dependent launch).
 //
 // A half-step needs everything the previous one wrote, so its CTAs can only
-// start working when that grid is complete; but they can be launched, placed on
-// their SMs and waiting by then.  Every half-step kernel begins with
-// pdl_begin(): wait for the previous grid (complete, its writes visible), then
-// allow the next one to be placed.  Nothing that a half-step writes may be
-// read before it, so the stages are read with ordinary loads: the read-only
-// path (__ldg) lets the compiler move a load above the wait.
+// start working when that grid is complete; but the launch itself is ready by
+// then.  Every half-step kernel begins with pdl_begin(), which waits for the
+// previous grid (complete, its writes visible).  Nothing that a half-step writes
+// may be read before it, and stages are not read through the read-only path
+// (__ldg), whose data must not change while the grid exists.
+//
+// No kernel asks for the next one to be placed early
+// (griddepcontrol.launch_dependents): its waiting CTAs would fill the slots that a
+// grid of less than one wave leaves free, unevenly over the SMs.  With the request
+// at the start of the kernel and without: FP64 Euler P = 3 at 2^15 cells 47.6 and
+// 33.7 us per half-step, FP32-mixed Euler P = 3 at 2^17 10.4 and 9.0 us (in pairs 8.4 and
+// 7.0), P = 2 at 370 000 cells 16.2 and 13.9; elsewhere the request gained 6 % at most
+// (FP64 advection P = 2 at 2^14 cells 6.0 and 6.3, FP32-mixed Euler P = 3 at 2^18 11.3 and
+// 11.6, at 2^22 117.2 and 117.5).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -16,7 +24,6 @@ namespace wcc {
 
 __device__ __forceinline__ void pdl_begin() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // kernel<<<grid, block, smem, stream>>>(args) with programmatic stream
