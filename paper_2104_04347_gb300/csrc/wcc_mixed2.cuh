@@ -401,8 +401,11 @@ constexpr int mixed2_smem_float2() {
 // own, where each plane's address is the same for the whole CTA up to the
 // thread's number (no 64-bit addition per access: 263 -> 253 us per half-step for
 // the batch of 768, 129.5 -> 127.9 us for 2^22 cells, Euler P = 3).  Scalar systems
-// (a third of the loads; Burgers P = 4 at 250 007 cells 7.7 -> 7.9 us with it) and the
-// cluster kernel, bound by the latency of one tile, do better with the shorter code.
+// (a third of the loads) take it from kLargeScalar cells on: Burgers P = 4 at 250 007
+// cells 7.25 us without and 7.35 with it, at 2^19 12.1 and 10.9, at 2^22 75.7 and
+// 69.1.  The cluster kernel, bound by the latency of one tile, does better with the
+// shorter code.
+constexpr long long kLargeScalar = 1 << 18;
 template <int SYS, int P, bool COMP, bool INNER = (SYS == EULER)>
 __device__ __forceinline__ void mixed_load_parents(const TileIO& io, ff2 (&ub)[nvars(SYS)],
                                                    f2 (&c)[nvars(SYS)][P + 1]) {
@@ -422,7 +425,7 @@ __device__ __forceinline__ void mixed_load_parents(const TileIO& io, ff2 (&ub)[n
             });
         });
     };
-    if (INNER && first >= 0 && first + 2 * kThreadsMixed <= io.n_old) {
+    if (INNER && (SYS == EULER || io.n_old >= kLargeScalar) && first >= 0 && first + 2 * kThreadsMixed <= io.n_old) {
         load(io.in32 + first, io.pitch, [&](const float* p) { return f2(load_once<SYS == EULER>(p + t), load_once<SYS == EULER>(p + t + kThreadsMixed)); });
     } else {
         const long long pa = parent_index(first + t, io.n_old, io.bc);
@@ -644,6 +647,8 @@ __device__ __forceinline__ float mixed_cell_speed(const ff2 (&ubn)[nvars(SYS)], 
     return fmaxf(va ? sp.x() : 0.f, vb ? sp.y() : 0.f);
 }
 
+// Scalar systems address their stores cell by cell: Burgers P = 1 at 2^20 cells 12.0 ->
+// 11.4 us, P = 2 at 2^22 43.7 -> 43.1; Euler does better with an address per plane.
 // New cells io.first_new + t (lane x, if va) and io.first_new + t +
 // kThreadsMixed (lane y, if vb) into the stage io.out32; returns the larger
 // of their speeds.
@@ -655,12 +660,18 @@ __device__ __forceinline__ float mixed_store(const TileIO& io, const ff2 (&ubn)[
     constexpr int K = P + 1;
     constexpr int NP = P + 2;
     const unsigned t = threadIdx.x;
-    float* tile = io.out32 + io.first_new;
+    float* tile = io.out32 + (SYS == EULER ? io.first_new : 0);
+    const long long ia = io.first_new + t, ib = ia + kThreadsMixed;
     f2 u0n[NV];
     f2 check(0.f);  // NaN / Inf in any stored value reaches this sum
     auto store = [&](float* p, f2 x) {
-        if (va) __stcs(p + t, x.x());
-        if (vb) __stcs(p + t + kThreadsMixed, x.y());
+        if constexpr (SYS == EULER) {
+            if (va) __stcs(p + t, x.x());
+            if (vb) __stcs(p + t + kThreadsMixed, x.y());
+        } else {
+            if (va) __stcs(p + ia, x.x());
+            if (vb) __stcs(p + ib, x.y());
+        }
     };
     sfor<0, NV>([&](auto V) {
         constexpr int v = decltype(V)::value;
@@ -687,7 +698,10 @@ __device__ __forceinline__ float mixed_store(const TileIO& io, const ff2 (&ubn)[
 // synchronises the block before rec is written again.  step() gives the
 // half-step's size; it is called after the parents' loads have been issued,
 // so that reading the device state does not delay them (the state's fields
-// decide a branch, which waits for them).
+// decide a branch, which waits for them).  Large scalar meshes at P >= 3 read the
+// state first: per half-step Burgers P = 3 at 2^22 cells 65.8 -> 62.3 us, advection
+// P = 4 69.7 -> 66.7, Burgers P = 4 69.1 -> 71.1 (2^19 cells: 9.6 -> 10.4, 10.3 ->
+// 10.9, 10.9 -> 11.1, which sets the line at 2^20).
 template <int SYS, int P, bool COMP, bool PARK = (P >= 3), bool SMALL = false, class Step>
 __device__ __forceinline__ void mixed_tile2(const TileIO& io, Step&& step, const StepArgs& args, float2* rec,
                                             float& speed, unsigned& err) {
@@ -697,8 +711,11 @@ __device__ __forceinline__ void mixed_tile2(const TileIO& io, Step&& step, const
     {
         ff2 ub[NV];
         f2 c[NV][K];
-        mixed_load_parents<SYS, P, COMP, SYS == EULER && !SMALL>(io, ub, c);
-        const StepSize& z = step();
+        const bool step_first = SYS != EULER && P >= 3 && !SMALL && io.n_old >= 4 * kLargeScalar;
+        StepSize z;
+        if (step_first) z = step();
+        mixed_load_parents<SYS, P, COMP, !SMALL>(io, ub, c);
+        if (!step_first) z = step();
         const ff2 lam2{f2(z.lam_hi), f2(COMP ? z.lam_lo : 0.f)};
         mixed_parent_records<SYS, P, COMP, PARK>(ub, c, lam2, args, rec);
     }

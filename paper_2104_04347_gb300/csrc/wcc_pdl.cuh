@@ -52,9 +52,10 @@ cudaError_t launch_pdl(void (*kernel)(A), dim3 grid, unsigned block, size_t smem
 // (load_once).  FP32-mixed Euler, P = 3, per half-step: 2^22 cells
 // (251 MB a stage) 125.5 -> 121.6 us, the batch of 768 meshes 248.0 -> 238.5 us
 // (246.2 from the direction, the rest from the loads), 2^20 cells in pairs
-// 23.2 -> 22.9 us.  Scalar systems (LARGE false: a third of the bytes, seldom more
-// than L2) keep one direction and plain loads: Burgers P = 4 at 250 007 cells
-// 7.6 us, 7.7 with both.
+// 23.2 -> 22.9 us.  Scalar systems (LARGE false: a third of the bytes) keep one
+// direction and plain loads, which is the better choice for P = 1 at every size
+// (Burgers at 2^22 cells, 67 MB a stage, 39.4 us, 40.8 with both) and up to 2^20 cells
+// above (P = 4 at 250 007 cells 7.0 us, 7.3 with both; at 2^22, 100 MB, 78.0 and 76.6).
 template <bool LARGE>
 __device__ __forceinline__ long long sweep_index(const void* in, const void* out, long long i, long long n) {
     return LARGE && in > out ? n - 1 - i : i;
