@@ -3,8 +3,10 @@
 // [row][col][var][q] (FP64) and the device planes.
 //
 // Device layout: plane (v, q) holds the Taylor coefficient e_kl = u_{kx,ly} /
-// (k! l!) of variable v (q = position of (k, l)) for every cell, row-major with `pitch` elements per row; planes are
-// `plane` elements apart.  T is double (FP64 path) or float (FP32 path).
+// (k! l!) of variable v (q = position of (k, l); FP64: of (3, 0) and (0, 3) the
+// derivative itself, see kept) for every cell, row-major with `pitch` elements per
+// row; planes are `plane` elements apart.  T is double (FP64 path) or float (FP32
+// path).
 //
 // The half-step kernel runs one CTA of TW threads per strip of TW - 1 new
 // columns and `rows_per_cta` new rows.  It marches up the strip: each step
@@ -343,7 +345,7 @@ template <int P, bool MX, class T, class Put>
 __device__ __forceinline__ void variable_to_planes(const unsigned long long* d, Put&& put) {
     if constexpr (sizeof(T) == 8) {
         unroll<nq(P)>([&](auto qc) {
-            constexpr double w = 1.0 / fact_q(qc);
+            constexpr double w = kept<d3>(qc) / fact_q(qc);
             const double x = __longlong_as_double((long long)d[qc]);
             put(qc, w == 1.0 ? x : x * w);
         });
@@ -376,8 +378,9 @@ template <int P, bool MX, class T, class Get>
 __device__ __forceinline__ void planes_to_variable(Get&& get, unsigned long long* d) {
     if constexpr (sizeof(T) == 8) {
         unroll<nq(P)>([&](auto qc) {
+            constexpr double w = fact_q(qc) / kept<d3>(qc);
             const double x = get(qc);
-            d[qc] = (unsigned long long)__double_as_longlong(fact_q(qc) == 1.0 ? x : x * fact_q(qc));
+            d[qc] = (unsigned long long)__double_as_longlong(w == 1.0 ? x : x * w);
         });
     } else {
         float e[nq(P)];

@@ -203,6 +203,18 @@ __device__ __forceinline__ void unroll(F&& f) {
     unroll_seq(f, std::make_integer_sequence<int, (N > 0 ? N : 0)>{});
 }
 
+// How a stage and a new cell hold coefficient (k, l): e_kl times this.  FP64 holds the
+// derivatives u_3x and u_3y themselves: 6 is the one k! l! that is not a power of two, and
+// multiplied by it and divided again a value would not always come back, while every
+// stage read back to the host loads again bit for bit.  (FP32 coefficients times 6 are
+// exact in the host's doubles.)
+template <class R>
+__host__ __device__ constexpr double kept(int k, int l) {
+    return std::is_same<R, d3>::value && (k == 3 || l == 3) ? 6.0 : 1.0;
+}
+template <class R>
+__host__ __device__ constexpr double kept(int q) { return kept<R>(qk_of(q), ql_of(q)); }
+
 // mean of xi^k over [0, 1/2]
 __host__ __device__ constexpr double half_mean(int k) { return pow2m(k) / (k + 1); }
 
@@ -218,7 +230,10 @@ __device__ __forceinline__ void parent_terms(const R (&q)[nvars(SYS)][nq(P)], R 
     R X[NV][P + 1][P + 1][P + 1];
     unroll<NV>([&](auto vc) {
         unroll<P + 1>([&](auto kc) {
-            unroll<P + 1 - kc>([&](auto lc) { X[vc][kc][lc][0] = q[vc][qidx(kc, lc)]; });
+            unroll<P + 1 - kc>([&](auto lc) {
+                constexpr double c = 1.0 / kept<R>(kc, lc);
+                X[vc][kc][lc][0] = WCC2D_TIMES(q[vc][qidx(kc, lc)], c);
+            });
         });
     });
     // time-averaged fluxes on the half lines through the centre, along x the
@@ -401,7 +416,7 @@ __device__ __forceinline__ void parent_terms(const R (&q)[nvars(SYS)][nq(P)], R 
             unroll<P + 1 - kc>([&](auto lc) {
                 constexpr int k = kc, l = lc;
                 if constexpr (k + l >= 2 && !(k == 1 && l == 1)) {
-                    const R w = cst<R>(0.25 * half_mean(k) * half_mean(l));
+                    const R w = cst<R>(0.25 * half_mean(k) * half_mean(l) / kept<R>(k, l));
                     if constexpr (!(k & 1) && !(l & 1)) a = fma(w, q[v][qidx(k, l)], a);
                     else if constexpr (!(l & 1)) p = fma(w, q[v][qidx(k, l)], p);
                     else if constexpr (!(k & 1)) s = fma(w, q[v][qidx(k, l)], s);
@@ -446,7 +461,8 @@ __device__ __forceinline__ void parent_terms(const R (&q)[nvars(SYS)][nq(P)], R 
 // (1 lower left, 2 lower right, 3 upper right, 4 upper left),
 //   (k+1) e_{k+1,l} = ((T_2 + T_3) - (T_1 + T_4))_{kl} / 2
 //       - sum_{s odd, t even, s+t >= 3} 2^{1-s-t} C(k+s, s) C(l+t, t) e_{k+s,l+t}
-// and the same along y.  dxy(k, l, dx, dy) gives the two differences.
+// and the same along y, each as a new cell keeps it (kept).  dxy(k, l, dx, dy) gives
+// the two differences.
 template <int P, int LOW, class R, class Diff>
 __device__ __forceinline__ void derivatives2d(Diff&& dxy, R (&D)[nq(P)]) {
     unroll<P + 1 - LOW>([&](auto dd) {
@@ -457,15 +473,16 @@ __device__ __forceinline__ void derivatives2d(Diff&& dxy, R (&D)[nq(P)]) {
             R dx, dy;
             dxy(std::integral_constant<int, qidx(k, l)>{}, dx, dy);
             // mixed derivatives are the mean of the two formulas
-            constexpr double wx = (l > 0 ? 0.5 : 1.0) / (k + 1), wy = (k > 0 ? 0.5 : 1.0) / (l + 1);
-            R ex = cst<R>(0.5 * wx) * dx, ey = cst<R>(0.5 * wy) * dy;
+            constexpr double wx = (l > 0 ? 0.5 : 1.0) / (k + 1) * kept<R>(k + 1, l),
+                             wy = (k > 0 ? 0.5 : 1.0) / (l + 1) * kept<R>(k, l + 1);
+            R ex = WCC2D_TIMES(dx, 0.5 * wx), ey = WCC2D_TIMES(dy, 0.5 * wy);
             unroll<r + 1>([&](auto sc) {
                 unroll<r + 1>([&](auto tc) {
                     constexpr int s = sc, t = tc;
                     if constexpr ((s & 1) && !(t & 1) && s + t >= 3 && s + t <= r) {
-                        ex = fma(cst<R>(-wx * 2.0 * pow2m(s + t) * binomd(k + s, s) * binomd(l + t, t)),
+                        ex = fma(cst<R>(-wx * 2.0 * pow2m(s + t) * binomd(k + s, s) * binomd(l + t, t) / kept<R>(k + s, l + t)),
                                  D[qidx(k + s, l + t)], ex);
-                        ey = fma(cst<R>(-wy * 2.0 * pow2m(s + t) * binomd(l + s, s) * binomd(k + t, t)),
+                        ey = fma(cst<R>(-wy * 2.0 * pow2m(s + t) * binomd(l + s, s) * binomd(k + t, t) / kept<R>(k + t, l + s)),
                                  D[qidx(k + t, l + s)], ey);
                     }
                 });
@@ -510,8 +527,14 @@ __device__ __forceinline__ void first_derivatives(R (&d)[nq(P)], const R (&vv)[4
     const R A = vv[2] - vv[0], B = vv[1] - vv[3];
     R ex = cst<R>(0.5) * (A + B), ey = cst<R>(0.5) * (A - B);
     if constexpr (P >= 3) {
-        ex = fma(cst<R>(-0.25), d[qidx(3, 0)] + d[qidx(1, 2)], ex);
-        ey = fma(cst<R>(-0.25), d[qidx(0, 3)] + d[qidx(2, 1)], ey);
+        if constexpr (is_f32<R>) {
+            ex = fma(cst<R>(-0.25), d[qidx(3, 0)] + d[qidx(1, 2)], ex);
+            ey = fma(cst<R>(-0.25), d[qidx(0, 3)] + d[qidx(2, 1)], ey);
+        } else {
+            constexpr double c = -0.25 / kept<R>(3, 0);
+            ex = fma(cst<R>(c), d[qidx(3, 0)], fma(cst<R>(-0.25), d[qidx(1, 2)], ex));
+            ey = fma(cst<R>(c), d[qidx(0, 3)], fma(cst<R>(-0.25), d[qidx(2, 1)], ey));
+        }
     }
     d[1] = ex;
     d[2] = ey;
@@ -520,7 +543,7 @@ __device__ __forceinline__ void first_derivatives(R (&d)[nq(P)], const R (&vv)[4
 // ----------------------------------------------------------------- limiter
 
 // Limiter of Sec. 3.2 for one scalar component in deviation form: d[1..] the
-// Taylor coefficients of u_0 (replaced by those of u_*) and the vertex
+// Taylor coefficients of u_0 as kept (replaced by those of u_*) and the vertex
 // values vv[0..3] at vertices 1..4 less the cell average ub, which the limiter
 // keeps (only the rounding of FP64's residuals depends on it).  FP64 follows the printed weights; in
 // FP32 the same weights are formed from ratios (every term divided by the
@@ -554,11 +577,11 @@ __device__ __forceinline__ bool limit_scalar(R (&d)[nq(P)], const R (&vv)[4], co
     // over q1 of d[q1] times an inner sum over q2 (independent chains)
     unroll<NQ - 1>([&](auto q1c) {
         constexpr int q1 = q1c + 1;
-        constexpr double c1 = beta_coef(P, qk_of(q1), ql_of(q1), qk_of(q1), ql_of(q1));
+        constexpr double c1 = beta_coef(P, qk_of(q1), ql_of(q1), qk_of(q1), ql_of(q1)) / (kept<R>(q1) * kept<R>(q1));
         R inner = WCC2D_TIMES(d[q1], c1);
         unroll<NQ>([&](auto q2) {
             if constexpr (q2 > q1) {
-                constexpr double c = 2.0 * beta_coef(P, qk_of(q1), ql_of(q1), qk_of(q2), ql_of(q2));
+                constexpr double c = 2.0 * beta_coef(P, qk_of(q1), ql_of(q1), qk_of(q2), ql_of(q2)) / (kept<R>(q1) * kept<R>(q2));
                 if constexpr (c != 0.0) inner = fma(cst<R>(c), d[q2], inner);
             }
         });
@@ -616,7 +639,9 @@ __device__ __forceinline__ bool limit_scalar(R (&d)[nq(P)], const R (&vv)[4], co
         } else {
             const R t0 = fma(d[qidx(3, 0)], d[qidx(3, 0)], d[qidx(0, 3)] * d[qidx(0, 3)]);
             const R t1 = fma(d[qidx(2, 1)], d[qidx(2, 1)], d[qidx(1, 2)] * d[qidx(1, 2)]);
-            tau = fma(cst<R>(36.0), t0, cst<R>(4.0) * t1);
+            constexpr double c = 36.0 / (kept<R>(3, 0) * kept<R>(3, 0));
+            if constexpr (c == 1.0) tau = fma(cst<R>(4.0), t1, t0);
+            else tau = fma(cst<R>(c), t0, cst<R>(4.0) * t1);
         }
         const R st = (half_sigma + half_sigma) * tau;
         if constexpr (!is_f32<R>) {
