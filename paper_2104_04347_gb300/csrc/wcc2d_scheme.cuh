@@ -142,13 +142,21 @@ __device__ __forceinline__ float sqrt_t(float x, float& inv) {
     return c;
 }
 __device__ __forceinline__ d3 sqrt_t(d3 x, d3& inv) { return wcc::sqrt_and_recip(x, inv); }
-// 1/sqrt(x) for a direction
-__device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
-__device__ __forceinline__ d3 rsqrt_t(d3 x) {
-    d3 inv;
-    (void)sqrt_t(x, inv);
-    return inv;
+// (a, b) / sqrt(x) for a direction
+__device__ __forceinline__ void over_root(float a, float b, float x, float& oa, float& ob) {
+    const float rn = rsqrtf(x);
+    oa = a * rn;
+    ob = b * rn;
 }
+__device__ __forceinline__ void over_root(d3 a, d3 b, d3 x, d3& oa, d3& ob) {
+    d3 ic;
+    const d3 c = sqrt_t(x, ic);
+    oa = wcc::quotient(a, c, ic);
+    ob = wcc::quotient(b, c, ic);
+}
+// a / b from rb = 1/b: FP64 rounded once
+__device__ __forceinline__ float over(float a, float, float rb) { return a * rb; }
+__device__ __forceinline__ d3 over(d3 a, d3 b, d3 rb) { return wcc::quotient(a, b, rb); }
 
 __device__ __forceinline__ float weight_pow(float x, const Law2D& law) {
     return law.alpha_is_two ? x * x : exp2f(law.alpha_f * log2f(x));
@@ -597,9 +605,9 @@ __device__ __forceinline__ bool limit_scalar(R (&d)[nq(P)], const R (&vv)[4], co
         if constexpr (!is_f32<R>) {
 #pragma unroll
             for (int m = 0; m < 5; ++m) w[m] = weight_pow(recip_t(beta[m] + eps), law);
-            const R is = recip_t(((w[0] + w[1]) + (w[2] + w[3])) + w[4]);
+            const R sum = ((w[0] + w[1]) + (w[2] + w[3])) + w[4], is = recip_t(sum);
 #pragma unroll
-            for (int m = 1; m < 5; ++m) w[m] = w[m] * is;
+            for (int m = 1; m < 5; ++m) w[m] = over(w[m], sum, is);
             w[0] = cst<R>(1.0) - ((w[1] + w[2]) + (w[3] + w[4]));
         } else {
             // every weight divided by that of the smallest denominator
@@ -654,11 +662,11 @@ __device__ __forceinline__ bool limit_scalar(R (&d)[nq(P)], const R (&vv)[4], co
             }
             if (law.alpha_is_two && wcc::exponent_of(st) + 32 <= least) return false;
 #pragma unroll
-            for (int m = 0; m < 5; ++m) w[m] = weight_pow(st * recip_t(den[m]), law);
+            for (int m = 0; m < 5; ++m) w[m] = weight_pow(wcc::quotient(st, den[m]), law);
             const R rest = (w[1] + w[2]) + (w[3] + w[4]);
-            const R is = recip_t((w[0] + cst<R>(1.0)) + rest);
+            const R sum = (w[0] + cst<R>(1.0)) + rest, is = recip_t(sum);
 #pragma unroll
-            for (int m = 1; m < 5; ++m) w[m] = w[m] * is;
+            for (int m = 1; m < 5; ++m) w[m] = over(w[m], sum, is);
             w[0] = cst<R>(1.0) - ((w[1] + w[2]) + (w[3] + w[4]));  // 1 when the others vanish
         } else {
             // divide every weight by (st / dmin)^alpha, dmin the smallest denominator
@@ -725,15 +733,11 @@ __device__ __forceinline__ bool limit_euler(R (&D)[4][nq(P)], const R (&ub)[4], 
     R gx = (gA + gB) * lamx, gy = (gA - gB) * lamy;  // (twice the gradient: only its direction counts)
     const R g2 = fma(gx, gx, gy * gy);
     R nx = cst<R>(1.0), ny = cst<R>(0.0);
-    if (positive(g2)) {
-        const R rn = rsqrt_t(g2);
-        nx = gx * rn;
-        ny = gy * rn;
-    }
+    if (positive(g2)) over_root(gx, gy, g2, nx, ny);
     const R gm1 = pick<R>(law.g1, law.g1_f), gamma = pick<R>(law.gamma, law.gamma_f);
     const R rho = ub[0];
     const R irho = recip_t(rho);
-    const R u = ub[1] * irho, v = ub[2] * irho;
+    const R u = over(ub[1], rho, irho), v = over(ub[2], rho, irho);
     const R hq2 = cst<R>(0.5) * fma(u, u, v * v);
     const R p = gm1 * fma(-rho, hq2, ub[3]);
     if (!positive(rho) || !positive(p)) return false;
@@ -741,8 +745,8 @@ __device__ __forceinline__ bool limit_euler(R (&D)[4][nq(P)], const R (&ub)[4], 
     // c and 1/c within an ulp of each other, so that the left and right
     // eigenvectors stay inverse to rounding (the projection and the
     // back-projection then cancel where the weights are linear)
-    const R c = sqrt_t(gamma * p * irho, ic);
-    const R H = (ub[3] + p) * irho;
+    const R c = sqrt_t(over(gamma * p, rho, irho), ic);
+    const R H = over(ub[3] + p, rho, irho);
     const R un = fma(u, nx, v * ny), ut = fma(v, nx, -(u * ny));
     if constexpr (!is_f32<R>) {
         // With X = (b_1/2) (q^2/2 d_0 - u d_1 - v d_2 + d_3), b_1 = (gamma - 1)/c^2, and
@@ -750,7 +754,7 @@ __device__ __forceinline__ bool limit_euler(R (&D)[4][nq(P)], const R (&ub)[4], 
         //   L d = (X - Y, d_0 - 2 X, n x (d_1, d_2) - u_t d_0, X + Y),
         //   R w = (s + w_1, u (s + w_1) + n_x m - n_y w_2, v (s + w_1) + n_y m + n_x w_2,
         //          H s + q^2/2 w_1 + u_t w_2 + u_n m),  s = w_0 + w_3, m = c (w_3 - w_0).
-        const R hic = cst<R>(0.5) * ic, b1h = (gm1 * hic) * ic, kx = nx * hic, ky = ny * hic, ku = un * hic;
+        const R cc = c * c, hic = cst<R>(0.5) * ic, b1h = cst<R>(0.5) * over(gm1, cc, recip_t(cc)), kx = nx * hic, ky = ny * hic, ku = un * hic;
         auto left = [&](R d0, R d1, R d2, R d3_, R (&w)[4]) {
             const R Xc = b1h * fma(-u, d1, fma(-v, d2, fma(hq2, d0, d3_)));
             const R Y = fma(kx, d1, fma(ky, d2, -(ku * d0)));
@@ -875,11 +879,11 @@ __device__ __forceinline__ R cfl_rate(const R* centre, const Law2D& law, R idx, 
     } else {
         const R rho = centre[0];
         if (!positive(rho)) return cst<R>(NAN);
-        const R irho = recip_t(rho), u = centre[1] * irho, v = centre[2] * irho;
+        const R irho = recip_t(rho), u = over(centre[1], rho, irho), v = over(centre[2], rho, irho);
         const R p = pick<R>(law.g1, law.g1_f) * fma(cst<R>(-0.5) * rho, fma(u, u, v * v), centre[3]);
         if (!positive(p)) return cst<R>(NAN);
         R ic;
-        const R c = sqrt_t(pick<R>(law.gamma, law.gamma_f) * p * irho, ic);
+        const R c = sqrt_t(over(pick<R>(law.gamma, law.gamma_f) * p, rho, irho), ic);
         return fma(fabs(u) + c, idx, (fabs(v) + c) * idy);
     }
 }

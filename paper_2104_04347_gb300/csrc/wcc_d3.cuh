@@ -83,6 +83,7 @@ __device__ __forceinline__ bool moderate(double x) {
 }
 static __device__ __noinline__ double recip_any(double x) { return 1.0 / x; }
 static __device__ __noinline__ double sqrt_any(double x) { return ::sqrt(x); }
+static __device__ __noinline__ double quotient_any(double a, double b) { return a / b; }
 
 // x with all 52 fraction bits set
 __device__ __forceinline__ bool fraction_full(double x) {
@@ -111,6 +112,12 @@ __device__ __forceinline__ d3 recip(d3 x) {
 __device__ __forceinline__ d3 quotient(d3 a, d3 b, d3 rb) {
     const d3 q = a * rb;
     return fma(fma(-q, b, a), rb, q);
+}
+
+// a / b for any operands
+__device__ __forceinline__ d3 quotient(d3 a, d3 b) {
+    if (moderate(a.v) && moderate(b.v)) return quotient(a, b, recip(b));
+    return d3::reg(quotient_any(a.v, b.v));
 }
 
 // the limiter's weights for an exponent other than 2
