@@ -332,7 +332,8 @@ __global__ void __launch_bounds__(256) stage_rate2d(const T* planes, long long p
 // whole sectors.  (One thread per cell, stepping through its cell's doubles:
 // 158 us to the planes and 527 us back at 1024 x 1024, FP32-mixed, P = 3; about
 // 110 and 190 us this way.)
-// FP32 stages are converted on the FP32 and integer pipes (wcc_convert.cuh).
+// FP32 coefficients are converted on the FP32 and integer pipes (wcc_convert.cuh);
+// what joins the FP32-mixed average and the point value is summed in FP64.
 constexpr int kConvCells = 64, kConvThreads = 256;
 
 // 1/(k! l!) and k! l! of position q
@@ -358,14 +359,15 @@ __device__ __forceinline__ void variable_to_planes(const unsigned long long* d, 
             else e[qc] = wcc::fast_two_sum(e[qc].hi, e[qc].lo);
         });
         if constexpr (MX) {
-            ff u = e[0];
+            double u = __longlong_as_double((long long)d[0]);
             if constexpr (P >= 2) {
-                constexpr wcc::ffc w = wcc::ffc_of(1.0 / 12.0);
-                u = wcc::ff_add(u, wcc::ff_mul_c(wcc::ff_add(e[qidx(2, 0)], e[qidx(0, 2)]), w));
+                u = ::fma(1.0 / 24.0, __longlong_as_double((long long)d[qidx(0, 2)]), u);
+                u = ::fma(1.0 / 24.0, __longlong_as_double((long long)d[qidx(2, 0)]), u);
             }
-            u = wcc::fast_two_sum(u.hi, u.lo);
-            put(0, u.hi);
-            put(-1, u.lo);
+            float hi, lo;
+            wcc::split_double(u, hi, lo);
+            put(0, hi);
+            put(-1, lo);
         } else {
             put(0, e[0].hi);
         }
@@ -390,14 +392,13 @@ __device__ __forceinline__ void planes_to_variable(Get&& get, unsigned long long
             d[i] = wcc::float_times_exact<(unsigned)fact_q(i)>(e[i]);
         });
         if constexpr (MX) {
-            ff u{get(0), get(-1)};
+            double u = __longlong_as_double((long long)wcc::float_times_exact<1>(get(0))) +
+                       __longlong_as_double((long long)wcc::float_times_exact<1>(get(-1)));
             if constexpr (P >= 2) {
-                constexpr wcc::ffc w = wcc::ffc_of(1.0 / 12.0);
-                u = wcc::ff_sub(u, wcc::ff_mul_c(wcc::two_sum(e[qidx(2, 0)], e[qidx(0, 2)]), w));
+                u = ::fma(-1.0 / 24.0, __longlong_as_double((long long)d[qidx(0, 2)]), u);
+                u = ::fma(-1.0 / 24.0, __longlong_as_double((long long)d[qidx(2, 0)]), u);
             }
-            d[0] = (unsigned long long)__double_as_longlong(
-                __longlong_as_double((long long)wcc::float_times_exact<1>(u.hi)) +
-                __longlong_as_double((long long)wcc::float_times_exact<1>(u.lo)));
+            d[0] = (unsigned long long)__double_as_longlong(u);
         } else {
             d[0] = wcc::float_times_exact<1>(get(0));
         }
@@ -666,9 +667,9 @@ __global__ void __launch_bounds__(TW, 4) halfstep2d_mx(const Step2D a) {
                 const ff hF = ffm_lazy(F[v], hx), hG = ffm_lazy(G[v], hy);
                 const float pr = par.p[v] + par.r[v], mr = par.p[v] - par.r[v];
                 ff c[4];
-                c[0] = ff_sum4(q4h, hF.hi, hG.hi, par.q[v] + pr, q4l + (hF.lo + hG.lo));
-                c[1] = ff_sum4(q4h, -hF.hi, hG.hi, par.q[v] - pr, q4l + (hG.lo - hF.lo));
-                c[2] = ff_sum4(q4h, -hF.hi, -hG.hi, -(par.q[v] + mr), q4l - (hF.lo + hG.lo));
+                c[0] = ff_sum4(q4h, hF.hi, hG.hi, par.q[v] + pr, (q4l + hF.lo) + hG.lo);
+                c[1] = ff_sum4(q4h, -hF.hi, hG.hi, par.q[v] - pr, (q4l - hF.lo) + hG.lo);
+                c[2] = ff_sum4(q4h, -hF.hi, -hG.hi, -(par.q[v] + mr), (q4l - hF.lo) - hG.lo);
                 c[3] = ff_rest3(ub[v], c[0], c[1], c[2]);
                 float2* r2 = reinterpret_cast<float2*>(r);
 #pragma unroll
