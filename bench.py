@@ -153,14 +153,26 @@ def peaks():
     return {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "sm_max_mhz": 2070.0}, "fallback"
 
 
-# FP64 operations the half-step kernel issues per cell-update (Euler, P = 3,
-# limiter on), counted from the executed DADD / DMUL / DFMA instructions (ncu
-# smsp__sass_thread_inst_executed_op_d{add,mul,fma}_pred_on.sum over one
-# launch at N = 2^20, DFMA counted as 2) divided by the cells of the launch.
-# Every operation is a three-register DFMA, additions and multiplications
-# too, so the figure measures the pipe's occupancy, not useful operations; the
-# limiter is left out where it does not act, most of this workload's cells.
-FP64_FLOPS_PER_CELL_UPDATE = (2 * 403418745 + 2105473) / 1048576.5
+# FP64 operations per cell-update of the half-step kernels, limiter on:
+# (additions, multiplications, fused multiply-adds), counted by an instrumented
+# build of the kernels' arithmetic type (one counter per operator) over four
+# half-steps of this workload at N = 2^16 after twenty.  The flops reported are the
+# useful ones, an addition or multiplication 1 and a fused one 2.  The kernels
+# issue every one of them as a three-register DFMA, so the FP64 pipe's
+# occupancy counts each as 2 and is reported under its own key.  The limiter's
+# weights are left out where they change nothing, most cells here.
+FP64_OPS = {1: (48.0, 78.1, 132.4), 2: (46.1, 83.2, 191.8), 3: (59.2, 107.4, 295.6), 4: (75.3, 137.6, 449.8),
+            5: (94.4, 171.8, 672.7), 6: (105.5, 221.2, 995.5)}
+
+
+def useful_flops(ops):
+    return ops[0] + ops[1] + 2 * ops[2]
+
+
+def issued_flops(ops):
+    return 2 * (ops[0] + ops[1] + ops[2])
+
+
 # DRAM bytes (read + write) of one launch at the bench size (N = 2^22), from
 # one ncu capture each (dram__bytes_read.sum + dram__bytes_write.sum, one
 # launch after three warm-up launches of the same kernel, graphs of 32
@@ -432,7 +444,7 @@ def time_solver(solver, stream, steps, warmup, barrier):
 def batch_bench(stream, steps, warmup, p3_rate, barrier):
     """The batched workload: 4096 independent Euler problems (N log-uniform in
     [256, 65536], P in {2, 3}, Riemann or density-wave data), FP32-mixed,
-    persistent launches in graphs of 32 half-steps, grid and pass depth (one
+    launches in graphs of 32 half-steps, grid and pass depth (one
     or two half-steps per launch) picked by the autotuner; the untuned batch
     (one half-step per launch, all resident CTAs) is timed beside it.
     Returns the batch line and the single-grid comparison."""
@@ -470,7 +482,7 @@ def batch_bench(stream, steps, warmup, p3_rate, barrier):
     single = 1.0 / ((cells[2] / ctot) / p2_rate + (cells[3] / ctot) / p3_rate)
     return {"workload": "euler1d-batch-4096-N256..65536-P2/3-riemann/density-wave", "value": value,
             "unit": "cell-updates/s", "ms_per_step": total_ms / steps, "steps": steps,
-            "cells_per_halfstep": per_step / HALFSTEPS_PER_STEP, "persistent_ctas": ctas,
+            "cells_per_halfstep": per_step / HALFSTEPS_PER_STEP, "ctas": ctas,
             "halfsteps_per_launch": depth, "pairs": pairs, "pair_fallbacks": fallbacks,
             "untuned_default_grid": value_one,
             "gpu_launches": launches, "single_grid_same_mix": single, "single_grid_p2": p2_rate,
@@ -570,12 +582,14 @@ def run_wcc(args, rank, world):
                                else "fallback 6.8 TB/s"),
                "bytes_per_cell_update": bpc, "kernel_ms": kernel_ms}
         if name == "fp64":
-            tf = FP64_FLOPS_PER_CELL_UPDATE * cells_per_launch / (kernel_ms * 1e-3) / 1e12
+            rate = cells_per_launch / (kernel_ms * 1e-3) / 1e12
+            tf = useful_flops(FP64_OPS[P]) * rate
             res["roofline"] = {"bound": "alu", "achieved": tf, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                                "frac": tf / FP64_PEAK_TFLOPS,
                                "traffic": FP64_TRAFFIC_2_22 if args.log2n == 22 else None,
                                "peak_source": "nominal GB300 FP64 1.25 TFLOP/s (recipe)",
-                               "flops_per_cell_update": FP64_FLOPS_PER_CELL_UPDATE, "kernel_ms": kernel_ms,
+                               "flops_per_cell_update": useful_flops(FP64_OPS[P]), "kernel_ms": kernel_ms,
+                               "fp64_pipe_occupancy": issued_flops(FP64_OPS[P]) * rate / FP64_PEAK_TFLOPS,
                                "hbm_frac": hbm["frac"]}
         else:
             if args.log2n == 22:
@@ -799,11 +813,11 @@ BYTES_2D_PER_CELL = {"fp32_mixed": 2 * 44 * 4, "fp32": 2 * 40 * 4, "fp64": 2 * 4
 # kernel, 64-thread strips) thread instructions of one launch at n = 1024
 # divided by the 1024^2 cells (FMA = 2 flops; min/max, compares and
 # conversions not counted; a paired FADD2 counts 2, a paired FFMA2 4).
-# FP32-mixed: 96-thread strips.  FP64: every operation is a DFMA, so its figure
-# is the pipe's occupancy.
+# FP32-mixed: 96-thread strips.  FP64: counted as FP64_OPS, at n = 512.
+FP64_OPS_2D = (438.7, 499.8, 1083.2)
 FLOPS_2D_PER_CELL = {"fp32_mixed": (1205938660 + 2 * 1043579606 + 424629952 + 2 * 12582912 + 4 * 155189248) / 1048576.0,
                      "fp32": (318283312 + 2 * 636306416 + 315836868 + 2 * 12582912 + 4 * 453492736 + 2 * 28827648) / 1048576.0,
-                     "fp64": 2 * 1967884767 / 1048576.0}
+                     "fp64": useful_flops(FP64_OPS_2D)}
 # DRAM bytes (read + write) of one launch per cell, same captures; scaled by
 # cells to the bench size.  The writes undercount the stored DOFs: part of
 # the output is still in L2 when the kernel ends.  FP32-mixed: one launch at
@@ -875,6 +889,8 @@ def two_d_bench(args):
             peak = FP64_PEAK_TFLOPS if name == "fp64" else fp32_peak
             r["arith"] = {"achieved_tflops": tf, "peak_tflops": peak, "frac": tf / peak,
                           "flops_per_cell": FLOPS_2D_PER_CELL[kind]}
+            if name == "fp64":
+                r["arith"]["fp64_pipe_occupancy"] = issued_flops(FP64_OPS_2D) * cells / per_launch_s / 1e12 / peak
         results[name] = r
     clk = clocks.stop()
     # CPU oracle on a bounded sample: the same vortex at 64 x 64, FP64, a few half-steps
@@ -915,14 +931,6 @@ def two_d_bench(args):
 # linear scheme (0.2116 at P = 5, 0.1851 at P = 6; Sec. 2.3), the bench's 0.2
 # below that.
 CFL_HIGH = {3: 0.2, 4: 0.2, 5: 0.16, 6: 0.14}
-# FP64 flops per cell-update of halfstep_fp64<EULER, P> (ncu DADD + DMUL +
-# 2 DFMA thread instructions of one launch over the launch's cells); P = 3 is
-# FP64_FLOPS_PER_CELL_UPDATE, P = 4..6 from one launch each at N = 2^20
-# (every operation a DFMA: the pipe's occupancy).
-FP64_FLOPS_HIGH = {3: None,
-                   4: (2105473 + 2 * 605019685) / 1048576.5,
-                   5: (2105473 + 2 * 884805957) / 1048576.5,
-                   6: (2105473 + 2 * 1271313777) / 1048576.5}
 
 
 def high_order_bench(args):
@@ -933,7 +941,6 @@ def high_order_bench(args):
 
     from paper_2104_04347_gb300 import inputs, wcc
 
-    FP64_FLOPS_HIGH[3] = FP64_FLOPS_PER_CELL_UPDATE
     stream = torch.cuda.Stream()
     clocks = ClockSampler()
     clocks.start()
@@ -968,9 +975,10 @@ def high_order_bench(args):
             k += 1
         row["oracle_cell_updates_per_s"] = sol.q.shape[0] * k / (time.perf_counter() - t0)
         row["oracle_cores"] = oracle.get_threads()
-        if FP64_FLOPS_HIGH[P]:
-            tf = FP64_FLOPS_HIGH[P] * cells / (ms / 1e3) / 1e12
-            row.update({"fp64_flops_per_cell": FP64_FLOPS_HIGH[P], "fp64_tflops": tf, "fp64_frac": tf / FP64_PEAK_TFLOPS})
+        rate = cells / (ms / 1e3) / 1e12
+        tf = useful_flops(FP64_OPS[P]) * rate
+        row.update({"fp64_flops_per_cell": useful_flops(FP64_OPS[P]), "fp64_tflops": tf, "fp64_frac": tf / FP64_PEAK_TFLOPS,
+                    "fp64_pipe_occupancy": issued_flops(FP64_OPS[P]) * rate / FP64_PEAK_TFLOPS})
         rows.append(row)
         print(json.dumps(row), flush=True)
     print(json.dumps({"clocks": clocks.stop()}), flush=True)
@@ -990,12 +998,8 @@ def high_order_bench(args):
 # (Euler).  Reported beside the kernels' own counts, not used as a roofline.
 ORACLE_FLOPS = {(1, 1): 93.0, (1, 2): 191.0, (1, 3): 314.0, (1, 4): 502.0,
                 (2, 1): 517.0, (2, 2): 847.0, (2, 3): 1252.0, (2, 4): 1852.0, (2, 5): 2725.0, (2, 6): 3934.0}
-# FP64 operations per cell-update the Burgers FP64 kernel executes
-# (halfstep_fp64<BURGERS, P>, limiter on): DADD + DMUL + 2 DFMA thread
-# instructions of one launch at N = 2^20 (ncu, profiles/burgers_halfstep.md)
-# over the launch's cells, e.g. P = 3: (1048577 + 2 x 80082825) / 2^20; every
-# operation is a DFMA, so the figures are the pipe's occupancy.
-BURGERS_FP64_FLOPS = {1: 83.17, 2: 101.43, 3: 153.75, 4: 242.32}
+# The Burgers FP64 kernel's operations per cell-update, as FP64_OPS.
+BURGERS_FP64_OPS = {1: (13.0, 16.0, 17.1), 2: (12.0, 19.1, 27.2), 3: (16.1, 26.1, 45.3), 4: (21.1, 39.3, 73.5)}
 BURGERS_CFL = {1: 0.4, 2: 0.3, 3: 0.25, 4: 0.2}
 
 
@@ -1010,7 +1014,7 @@ def burgers_bench(args):
     write of the state per launch: 16 (P + 1) B in FP64, 2 (8 + 4 P) B in
     FP32-mixed, half of that per cell-update with two half-steps per launch)
     and, for FP64, the fraction of the FP64 peak at the kernel's executed
-    FP64 operations (BURGERS_FP64_FLOPS);
+    FP64 operations (BURGERS_FP64_OPS);
     time to 2 t_s (past the shock) for N <= 2^18; and the oracle on the host
     cores on a bounded sample (N = 2^14, CFL half-steps for about
     cpu_seconds / 8 per degree)."""
@@ -1060,8 +1064,9 @@ def burgers_bench(args):
                        "bytes_per_cell_update": bpc, "hbm_gbs": bpc * rate / 1e9,
                        "hbm_frac": bpc * rate / 1e9 / pk["hbm_gbs"], "time_to_2ts": tts}
                 if prec == wcc.FP64:
-                    tf = BURGERS_FP64_FLOPS[P] * rate / 1e12
-                    row.update({"fp64_flops_per_cell_update": BURGERS_FP64_FLOPS[P],
+                    tf = useful_flops(BURGERS_FP64_OPS[P]) * rate / 1e12
+                    row.update({"fp64_flops_per_cell_update": useful_flops(BURGERS_FP64_OPS[P]),
+                                "fp64_pipe_occupancy": issued_flops(BURGERS_FP64_OPS[P]) * rate / 1e12 / FP64_PEAK_TFLOPS,
                                 "oracle_flops_per_cell_update": ORACLE_FLOPS[(1, P)], "fp64_tflops": tf,
                                 "fp64_frac": tf / FP64_PEAK_TFLOPS})
                 rows.append(row)
