@@ -67,8 +67,6 @@ __device__ __forceinline__ int parent_index(int j, int n_old, int bc) {
     return j < 0 ? 0 : (j > n_old - 1 ? n_old - 1 : j);
 }
 
-// Reads parent records from the ring: vertex r = 0..3 is parent column t
-// (r = 0, 3) or t + 1 (r = 1, 2) of the lower (r = 0, 1) or upper row.
 // Compute type of a stage type, and values between the two.
 template <class T>
 using compute_t = std::conditional_t<sizeof(T) == 8, d3, float>;
@@ -77,6 +75,8 @@ __device__ __forceinline__ d3 from_memory(double x) { return d3::reg(x); }
 __device__ __forceinline__ float to_memory(float x) { return x; }
 __device__ __forceinline__ double to_memory(d3 x) { return x.v; }
 
+// Reads parent records from the ring: vertex r = 0..3 is parent column t
+// (r = 0, 3) or t + 1 (r = 1, 2) of the lower (r = 0, 1) or upper row.
 template <class T, int TW, int NV, int NQ1>
 struct RingReader {
     using R = compute_t<T>;
@@ -173,9 +173,9 @@ constexpr int min_ctas2d() {
     return sizeof(T) == 4 ? 4 : 1;
 }
 
-// The FP64 kernel is bound by the FP64 pipe: Euler P = 3 issues about 2100 FP64
+// The FP64 kernel is bound by the FP64 pipe: Euler P = 3 issues about 2020 FP64
 // instructions per cell, all three-register DFMAs (about 3000 of every form in
-// the derivative form with IEEE divisions): 192 x 192 0.42 -> 0.25 ms per
+// the derivative form with the compiler's divisions): 192 x 192 0.42 -> 0.27 ms per
 // half-step.  The FP32 kernels are bound by issue and dependency latency at 12 to
 // 16 warps per SM.
 template <int SYS, int P, class T, int TW>

@@ -44,8 +44,6 @@ __host__ __device__ constexpr int qk_of(int q) { return qdeg(q) - ql_of(q); }
 __host__ __device__ constexpr double factd(int n) { return n <= 1 ? 1.0 : n * factd(n - 1); }
 __host__ __device__ constexpr double binomd(int n, int k) { return factd(n) / (factd(k) * factd(n - k)); }
 __host__ __device__ constexpr double pow2m(int n) { return n <= 0 ? 1.0 : 0.5 * pow2m(n - 1); }  // 2^-n
-__host__ __device__ constexpr double sgnd(int k) { return (k & 1) ? -1.0 : 1.0; }              // (-1)^k
-__host__ __device__ constexpr double ipow(double x, int n) { return n <= 0 ? 1.0 : x * ipow(x, n - 1); }
 
 // mean of xi^e over [-1/2, 1/2]
 __host__ __device__ constexpr double moment(int e) { return (e & 1) ? 0.0 : pow2m(e) / (e + 1); }
@@ -213,9 +211,9 @@ __device__ __forceinline__ void unroll(F&& f) {
 
 // How a stage and a new cell hold coefficient (k, l): e_kl times this.  FP64 holds the
 // derivatives u_3x and u_3y themselves: 6 is the one k! l! that is not a power of two, and
-// multiplied by it and divided again a value would not always come back, while every
-// stage read back to the host loads again bit for bit.  (FP32 coefficients times 6 are
-// exact in the host's doubles.)
+// a value multiplied by it and divided again does not always come back, whereas a
+// stage read back to the host has to load again bit for bit.  (FP32 coefficients
+// times 6 are exact in the host's doubles.)
 template <class R>
 __host__ __device__ constexpr double kept(int k, int l) {
     return std::is_same<R, d3>::value && (k == 3 || l == 3) ? 6.0 : 1.0;
@@ -1017,3 +1015,5 @@ __device__ __forceinline__ void linear_cell_mx(const Rd& rd, float (&D)[nvars(SY
 }
 
 }  // namespace wcc2d
+
+#undef WCC2D_TIMES
