@@ -506,8 +506,9 @@ int step_pairs(wcc_ctx* h, long long nsteps, double cfl) {
         h->tb_fallbacks += 1;
         h->cur = cur0 ^ (int)(done_pairs & 1);
         h->steps = st.step;
-        const unsigned e = st.err & ~ERR_CFL;
-        WCC_CHECK(h, cudaMemcpy(&h->st->err, &e, sizeof e, cudaMemcpyHostToDevice));
+        // (no other bit is set, read_state would have returned; on the handle's
+        // stream: a copy on the default stream could land after the half-steps below)
+        WCC_CHECK(h, cudaMemsetAsync(&h->st->err, 0, sizeof st.err, h->stream));
         for (int k = 0; k < 2; ++k)
             if ((rc = enqueue_one(h, cfl, 0.0)) != WCC_OK) return rc;
         pairs -= done_pairs + 1;

@@ -384,7 +384,10 @@ int do_step_pairs(wcc_batch_ctx* b, long long nsteps, double cfl) {
         std::vector<DevState> st;
         if ((rc = read_states(b, st)) != WCC_OK) return rc;
         for (auto& x : st) x.err &= ~ERR_CFL;
-        WCC_BCHECK(b, cudaMemcpy(b->d_st, st.data(), sizeof(DevState) * b->count, cudaMemcpyHostToDevice));
+        // on the batch's stream: a copy on the default stream could land after the
+        // half-steps below and put the states back
+        WCC_BCHECK(b, cudaMemcpyAsync(b->d_st, st.data(), sizeof(DevState) * b->count, cudaMemcpyHostToDevice, b->stream));
+        WCC_BCHECK(b, cudaStreamSynchronize(b->stream));
         const long long done_pairs = (st[0].step - steps0) / 2;
         b->tb_pairs += done_pairs;
         b->tb_fallbacks += 1;
