@@ -197,9 +197,13 @@ int ensure_hist(wcc_batch_ctx* b, long long need) {
     b->bytes += (cap - b->hist_cap) * b->count * (long long)sizeof(double);
     b->d_hist = nh;
     b->hist_cap = cap;
-    if (b->gexec) {
+    if (b->gexec) {  // captured launches hold the old pointer
         cudaGraphExecDestroy(b->gexec);
         b->gexec = nullptr;
+    }
+    if (b->gexec_tb) {
+        cudaGraphExecDestroy(b->gexec_tb);
+        b->gexec_tb = nullptr;
     }
     return WCC_OK;
 }
