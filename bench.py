@@ -1130,7 +1130,7 @@ def advection_config(args):
            "l1_vs_exact": float(np.mean(np.abs(q[:, 0, 0] - exact))),
            "max_vs_oracle": float(np.max(np.abs(q - sol.q))),
            "oracle_seconds": osecs, "oracle_cell_updates_per_s": 200 * len(dts) / osecs, "oracle_cores": 1,
-           "note": "200 cells: the GPU run is bound by launch latency, one launch per half-step"}
+           "note": "200 cells: the GPU run is bound by the latency of a half-step, up to 256 per launch of one cluster"}
     print(json.dumps(row), flush=True)
 
 

@@ -921,7 +921,7 @@ int wcc_step_until(wcc_handle h, double t_end, double cfl, int64_t* nsteps_taken
     const int chunk = h->opt.graph_chunk >= 2 ? h->opt.graph_chunk : 2;
     // A mesh that one cluster holds marches to t_end in it: the kernel applies
     // the rule below before every half-step (advection, 200 cells, 800 half-steps:
-    // 2.8 ms; 7.0 ms in graphs with a wait for the device state after each and, for
+    // 3.1 ms; 7.0 ms in graphs with a wait for the device state after each and, for
     // the last 128 half-steps, after every half-step).
     while (clustered(h) && h->opt.tb_depth == 1) {
         const double dt = next_dt(s);

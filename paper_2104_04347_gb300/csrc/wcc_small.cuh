@@ -17,8 +17,8 @@
 // (wcc_step_until's rule, decided here by every CTA from the same numbers).
 //
 // Measured per half-step, one launch each in graphs of 32 / one cluster:
-// advection P = 2 FP64, 200 cells (2 CTAs) 6.6 / 3.5 us; Euler P = 3 FP32-mixed, 2000
-// cells (8 CTAs) 6.45 / 3.2 us; Euler P = 3 FP64, 2001 cells (16 CTAs) 21.0 / 18.0 us
+// advection P = 2 FP64, 200 cells (2 CTAs) 7.1 / 3.8 us; Euler P = 3 FP32-mixed, 2000
+// cells (8 CTAs) 6.3 / 3.2 us; Euler P = 3 FP64, 2001 cells (16 CTAs) 22.7 / 19.5 us
 // (its FP64 chain alone takes 15).  The rule takes the cluster wherever one holds
 // the mesh, up to 16 tiles (2032 cells in FP64 and 4080 in FP32-mixed), and the
 // options do not ask for the tile kernels.
